@@ -437,86 +437,146 @@ void host_apply_plan(const PackedHost& ph, const ApplyPlan& plan, int fes, bool 
 // whole sweep (Alg. 3 / Alg. 4, flattened as for the cooperative kernel) for
 // its own one or two right-hand sides, so no CTA waits on another.  The
 // program is cut into
-//   * resident runs: subtrees whose vector rows and butterfly state fit the
-//     CTA's shared-memory window (their first group loads the rows, their
-//     last writes them back);
+//   * resident runs: subtrees whose vector rows and live butterfly state fit
+//     the CTA's shared-memory window (their first group loads the rows, their
+//     last writes them back).  A butterfly's stage is dead once the next one
+//     has read it, so a run needs its rows plus twice the largest stage;
 //   * global phases: the stages of the large butterflies, reading and
 //     writing the vector rows and a CTA-private butterfly state in global
-//     memory (each batch first gathers its distinct inputs into its warp's
+//     memory (each batch first gathers its ops' inputs into its warp's
 //     slice of the window, which is free between runs).
-// Every butterfly phase is a sparse product in row form (one output row =
-// an output slot and a list of (input, coefficient) entries: the ID's
-// identity entries, the T or S entries, conjugated and negated as the op
-// requires); sweep-leaf phases are the packed triangles of the exact subtree
-// inverse, applied in place.  The schedule is a sequence of staging groups,
-// one bulk copy each: a header, a phase table, the batch descriptors, the
-// batches' data.  A group holds several consecutive small phases of a resident
-// run (a barrier among the compute warps after each), or one part of a large
-// phase (the phase's last part ends with the barrier); a triangle is a group of
-// its own.  A resident run is executed by the first kSwChain compute warps
-// alone (their own barrier between phases; the other warps wait for the run's
-// end), which keeps the per-phase instruction overhead of this dependent chain
-// small; a global phase part's batches go round-robin to all compute warps.
+// Every op of a butterfly phase is written out as a dense block: the ID's
+// identity entries, the T or S entries (conjugated and negated as the op
+// requires) and zeros, over the op's inputs, which stand side by side in the
+// window (a stage is stored in the order in which the next one reads it) or in
+// the gathered slice.  So a row needs no index per entry, only where its inputs
+// start, and neighbouring entries can be multiplied in pairs (packed FP32).
+// Consecutive stages of a butterfly are multiplied out on the host where that is
+// cheaper than one more dependent phase.  Sweep-leaf phases are the triangles of the exact subtree inverse, applied in
+// place.  The schedule is a sequence of staging groups, one bulk copy each: a
+// header, a phase table, the batch descriptors, the batches' data.  A group
+// holds several consecutive small phases of a resident run, or one part of a
+// large phase; a triangle is a group of its own, and so is every batch of a global
+// phase, which belongs to one compute warp (the phase's groups in turn): a warp waits
+// only for the groups it works on.  A resident
+// phase of at most kSwSetTiles tiles belongs to one of two sets of kSwSet warps, in turn: while one
+// set computes, the other has already fetched its next tile's coefficients and
+// waits only for the inputs (hand-over by bar.arrive / bar.sync).  Larger phases
+// and triangles are taken by all compute warps, with a barrier of all before and
+// after.
+// Rows are laid out in tiles of 32 lanes: a row takes 2^glog neighbouring lanes,
+// each with the same even number of neighbouring inputs.
 // ---------------------------------------------------------------------------
-constexpr int kSwWarps = 12;                 // compute warps (one more warp stages the groups)
-constexpr int kSwChain = 8;                  // compute warps that execute the resident runs
+constexpr int kSwWarps = 16;                 // compute warps (one more warp stages the groups)
+constexpr int kSwSet = kSwWarps / 2;         // warps of a set
+constexpr int kSwSetTiles = 3 * kSwSet;      // resident phases of at most this many tiles go to the sets in turn
 constexpr int kSwWinBytes = 96 * 1024;       // resident window: rows + state of a run
-constexpr int kSwRingBytes = 104 * 1024;     // staging ring of group images
-constexpr int kSwPartBytes = 16 * 1024;      // partial sums of a triangle product
+constexpr int kSwRingBytes = 128 * 1024;     // staging ring of group images
 constexpr int kSwMaxCols = 2;                // right-hand sides per CTA
 constexpr int kSwWinSlots = kSwWinBytes / (kSwMaxCols * 8);   // window slots (complex-FP32 entries per column)
-constexpr int kSwGather = kSwWinSlots / (2 * kSwWarps);       // gathered inputs of a global batch (half a warp's
-                                                              // slice: the next batch's gather fills the other half)
-constexpr int kSwBatchBytes = 8 * 1024;      // target data bytes of one resident batch
-constexpr int kSwGlobBytes = 6 * 1024;       // target data bytes of one global batch
-constexpr int kSwGroupBytes = 32 * 1024;     // target bytes of a group
+constexpr int kSwGather = kSwWinSlots / (2 * kSwWarps);       // gathered inputs of a global batch (a warp's slice: as
+                                                              // gathered, and regrouped in pairs)
+constexpr int kSwGroupBytes = 40 * 1024;     // target bytes of a group
 constexpr int kSwMaxPhases = 64;             // phases of one group
+constexpr int kSwFlight = 64;                // slots of groups (arrival and release barriers)
+// Groups in flight.  A compute warp may wait for a group up to 2 kSwWarps - 1 further on than
+// the last one it has seen; with this limit the slot's previous group has been consumed by
+// then, so that the parity waited for is the slot's next one.
+constexpr int kSwAhead = kSwFlight - 2 * kSwWarps;
 constexpr int32_t kSwAcc = (int32_t)0x80000000;  // output slot flag: add to the output instead of overwriting
 enum SwGroupFlag : int32_t {
-  SWG_RES = 4,      // group: batches on the window (int16 window slots)
-  SWG_BEGIN = 8,    // group: load window rows [beg_lo, beg_hi) first
-  SWG_ENDRUN = 16,  // group: write window rows [end_lo, end_hi) back after its last phase
+  SWG_RES = 4,      // group: batches on the window
+  SWG_BEGIN = 8,    // group: load the window rows of vector rows [beg_lo, beg_hi) first
+  SWG_ENDRUN = 16,  // group: write vector rows [end_lo, end_hi) back after its last phase
 };
 enum SwPhaseFlag : int32_t {
   SWP_END = 1,      // the phase ends with this part: barrier among the compute warps
   SWP_TRI = 2,      // one triangle batch, taken by all compute warps
-  SWP_UPPER = 4     // triangle: upper
+  SWP_UPPER = 4,    // triangle: upper
+  // resident phases: who computes (all compute warps, or set 0 / 1), and the barrier after it
+  // (SWP_HAND: the next phase belongs to the other set and waits for this one only; else all warps meet)
+  SWP_ALL = 8,
+  SWP_SET1 = 16,
+  SWP_HAND = 32
 };
+// SwPhase::flags, upper bits: the phase's first descriptor in its group, and the warp that
+// takes its first tile (the parts of a phase spread over several groups continue the round)
+constexpr int kSwPhaseBase = 8, kSwBaseMask = 0xfff, kSwPhaseWarp = 20;
 struct SwGroup {     // one bulk copy
   int64_t img;       // byte offset of the group image
   int32_t bytes;     // multiple of 16
+  int32_t off;       // its place in the staging ring
+  int32_t need;      // groups [0, need) must be consumed before it may be copied there
   int32_t pad;
 };
+static_assert(sizeof(SwGroup) == 24, "group record");
 struct SwGroupHdr {  // first 32 bytes of a group image; then nph phase entries (8 bytes)
   int32_t nph, flags;
   int32_t beg_lo, beg_hi, end_lo, end_hi;
   int32_t off_desc;  // byte offset of the descriptors (all phases' batches in order)
-  int32_t aux;       // first group of a run (SWG_BEGIN): the run's group count; global
-                     // group: the compute warp that takes its first batch
+  int32_t aux;       // first group of a run (SWG_BEGIN) or of a global phase: its group count
 };
 struct SwPhase {
   int32_t nb, flags;
 };
-// Batch descriptor; offsets relative to the batch start.  Row form: out[nrows]
+// Window rows: leaf by leaf, each leaf's rows from an even slot (an odd leaf size
+// leaves one slot unused per leaf).  sw_row_slot: slot of local row i.
+HB_HD inline int32_t sw_leaf_stride(int32_t n0) { return n0 + (n0 & 1); }
+HB_HD inline int32_t sw_row_slot(int32_t i, int32_t n0) { return (n0 & 1) ? i / n0 * (n0 + 1) + i % n0 : i; }
+// Batch descriptor; offsets relative to the batch start.  Rows: out[nrows]
 // (int32 slot | kSwAcc; window slot for resident batches, else a global slot: a
-// vector row r < n or n + a state entry), e0[nrows + 1], coef[nent] (complex, the
-// factor's precision), in[nent] (int16: window slot, or position in the gather
-// list), gl[ngl] (int32 global slots of the distinct inputs, global batches
-// only).  Triangle: a packed lower triangle of order nrows, column by column
-// (rows c..s-1 of column c), applied in place to window rows a0 .. a0 + nrows - 1;
-// an upper triangle U is stored reversed (stored (r, c) = U(s-1-r, s-1-c), with
-// SWP_UPPER: stored row / column i stands for window row a0 + s-1-i).
+// vector row r < n or n + a state entry).  A tile is 32 lanes with elen (even)
+// entries each: in[32] (int16, even: the lane's first input, a window slot or a
+// position in the slice) and coef[32 elen], entry e of lane l at sw_pos(e, l) from
+// the tile's first: entries 2i, 2i + 1 of a lane adjacent, as (re, re, im, im).
+// A resident batch is one tile: out at 0, in at kSwTileIn, coef at kSwTileCoef.  A
+// global batch has nt = ceil(nrows >> (5 - glog)) tiles: tile t's lanes at
+// in[32 t], its entries from 32 e0[t] to 32 e0[t + 1] (int32 e0[nt + 1]); gl[ngl]
+// (int32 global slots of the slice's entries, -1 a zero; ngl even); a0 > 0: the rows
+// add to their outputs' old values, entries a0, a0 + 1, ... of the slice.
+// Triangle of order s = nrows, applied in place to the window rows from slot a0 on.
+// It is stored as a lower one, by column pairs p.  Lower triangle: stored row r = row
+// r, pair p = columns 2p, 2p + 1.  Upper (SWP_UPPER): stored row r = row s-1-r, pair p
+// = columns s-2-2p, s-1-2p.  Entries outside the triangle are zero.  Rows j and s-1-j
+// form a row pair (together s / 2 + 1 column pairs); four row pairs are one warp's
+// work (sw_tri_warp): n1 steps for the rows s-1-j, then n0 for the rows j, a step =
+// four row pairs x four neighbouring column pairs, (re, re, im, im) each.  The data:
+// kSwTriTab bytes with (first step << 16 | n1 << 8 | n0) of each warp, then the steps.
 struct SwDesc {
   int32_t off;       // byte offset of the batch inside the group image
+  int16_t elen;      // resident tile: entries per lane (even)
+  int8_t glog;       // log2 of the lanes that share one row (reduced by shuffles)
+  int8_t trows;      // resident tile: its rows
   int32_t nrows, nent, ngl;
   int32_t a0;
   int32_t off_e0, off_coef, off_in, off_gl;
-  int16_t glog;      // log2 of the lanes that share one row (reduced by shuffles)
-  int16_t pad;
 };
 static_assert(sizeof(SwGroupHdr) == 32, "group header");
 static_assert(sizeof(SwPhase) == 8, "phase entry");
 static_assert(sizeof(SwDesc) == 40, "batch descriptor");
+constexpr int kSwTileIn = 32 * 4, kSwTileCoef = kSwTileIn + 32 * 2;
+HB_HD inline int sw_pos(int e, int lane) { return (e >> 1) * 64 + lane * 2 + (e & 1); }
+constexpr int kSwTriTab = 256;
+struct SwTriWarp {
+  int n1, n0;
+};
+HB_HD inline int sw_tri_len(int r) { return r / 2 + 1; }   // column pairs of stored row r
+HB_HD inline bool sw_tri_live(int s, int j, bool hi) { return hi ? 2 * j <= s - 1 : 2 * j < s - 1; }   // row s-1-j / row j of pair j
+inline int sw_tri_warps(int s) { return ((s + 1) / 2 + 3) / 4; }
+inline SwTriWarp sw_tri_warp(int s, int v) {
+  SwTriWarp w{0, 0};
+  for (int j = 4 * v; j < 4 * v + 4; ++j) {
+    if (sw_tri_live(s, j, true)) w.n1 = w.n1 > (sw_tri_len(s - 1 - j) + 3) / 4 ? w.n1 : (sw_tri_len(s - 1 - j) + 3) / 4;
+    if (sw_tri_live(s, j, false)) w.n0 = w.n0 > (sw_tri_len(j) + 3) / 4 ? w.n0 : (sw_tri_len(j) + 3) / 4;
+  }
+  return w;
+}
+inline int sw_tri_steps(int s) {
+  int n = 0;
+  for (int v = 0; v < sw_tri_warps(s); ++v) n += sw_tri_warp(s, v).n1 + sw_tri_warp(s, v).n0;
+  return n;
+}
+inline int sw_tiles(int nrows, int glog) { return (nrows + (32 >> glog) - 1) / (32 >> glog); }
 struct SwSched {
   std::vector<SwGroup> groups;
   std::vector<uint8_t> image;

@@ -8,35 +8,36 @@
 // one or two right-hand sides and never waits on another CTA:
 //   * a producer warp streams the schedule's group images (host-built, see
 //     hb_swsched.cpp: a header, batch descriptors, the batches' data) into a
-//     shared-memory ring with one cp.async.bulk each, as far ahead as the
-//     ring allows -- the factor data never depends on the vectors, and the
-//     compute warps find every record they need in the ring;
-//   * resident runs (subtrees whose rows and butterfly state fit the 96 KB
+//     shared-memory ring with one cp.async.bulk each.  Every group's place in the
+//     ring, and the groups that must be consumed before it may be copied there, are
+//     fixed by the host, so 32 lanes issue 32 groups without any bookkeeping (a lane
+//     that allocated ring space and looked at every release took about a thousand
+//     cycles per group, which bounded the kernel);
+//   * resident runs (subtrees whose rows and live butterfly state fit the 96 KB
 //     window) start by loading their rows into shared memory and end by
 //     writing them back; inside them every phase reads and writes the window;
 //   * global phases (stages of the large butterflies) read and write the
-//     vector rows and a CTA-private butterfly state in global memory: a batch
-//     first gathers its distinct inputs into its warp's slice of the window
-//     (free between runs) in one round trip;
-//   * the resident runs -- the long dependent chain -- are executed by eight
-//     chain warps (two per scheduler) with their own barrier: a phase's rows
-//     are spread over eight warps, and a sweep leaf's columns over 256 threads,
-//     while the per-phase overhead is paid eight times, not twelve; the other
-//     compute warps wait for the run's end; a global phase's batches go
-//     round-robin to all twelve compute warps;
-//   * a butterfly phase is a sparse product in row form; in a batch, groups of
-//     2^glog lanes share a row (entries strided over the lanes, then a shuffle
-//     reduction), so that short dot products do not serialise on one lane;
-//   * a sweep-leaf phase (packed triangle, in place on the window rows) is
-//     taken by all chain warps: pairs of rows (j, s-1-j) times column groups,
-//     four independent accumulation chains, partial sums, a barrier, the
-//     reduction written back.
-// Consecutive phases are separated by one named barrier among the compute
-// warps; the groups of one phase are not.  Every wait is bounded; a warp whose
-// wait gives up stops computing but still meets the barriers up to the end of
-// the phase, where all compute warps learn of it and stop; the factor's error
-// flag is raised (reported by hb_status / the solvers) and the CTA returns
-// after a second bounded wait for its copies still in flight.
+//     vector rows and a CTA-private butterfly state in global memory; every batch
+//     belongs to one warp, which gathers its inputs (cp.async, the next batch's in
+//     flight while one is computed) and never touches the other warps' groups;
+//   * an op of a butterfly phase is a dense block over neighbouring inputs.  The
+//     window holds entry pairs as (re, re, im, im), so 16 bytes of coefficients and 16
+//     of inputs give two complex multiply-adds in four packed FP32 instructions, with
+//     no index per entry;
+//   * consecutive stages of a butterfly are multiplied out on the host where that is
+//     cheaper than one more dependent phase (the phases of the semicircle's sweep at
+//     N = 65,536: 3,058 without, 1,699 with);
+//   * the resident phases alternate between two sets of eight warps: while one set
+//     computes, the other has its next coefficients in registers and waits only for
+//     the inputs; large phases and the sweep leaves are taken by all sixteen.
+// What bounds it is the dependent chain of one CTA: a phase costs 1,000 to 2,000
+// cycles (descriptor and coefficient fetch, the inputs' round trip, shuffles, a
+// barrier), far above its share of the 9 B/clk of staged data.
+// Every wait is bounded; a warp whose wait gives up stops computing but still meets
+// the barriers up to the end of its unit (a run, a global phase), where all compute
+// warps learn of it and stop; the factor's error flag is raised (reported by
+// hb_status / the solvers) and the CTA returns after a second bounded wait for its
+// copies still in flight.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -50,11 +51,10 @@ namespace hb {
 namespace {
 
 constexpr int kSwThreads = (kSwWarps + 1) * 32;
-// at most four warps per scheduler: every thread may hold 128 registers
-static_assert((kSwWarps + 1 + 3) / 4 * 128 * 32 <= 16384, "registers per scheduler");
-constexpr int kSwSlots = 64;   // groups in flight per CTA
-constexpr int kSwSmem = kSwRingBytes + kSwWinBytes + kSwPartBytes;
-static_assert(kSwSmem <= 224 * 1024, "dynamic shared memory of the column-partitioned sweep");
+// at most five warps per scheduler: every thread may hold 96 registers
+static_assert((kSwWarps + 1 + 3) / 4 * 96 * 32 <= 16384, "registers per scheduler");
+constexpr int kSwSmem = kSwRingBytes + kSwWinBytes;   // ring | window
+static_assert(kSwSmem <= 225 * 1024, "dynamic shared memory of the column-partitioned sweep");
 
 __device__ __forceinline__ unsigned su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mb_init(uint64_t* b, unsigned count) {
@@ -66,6 +66,9 @@ __device__ __forceinline__ void mb_inval(uint64_t* b) {
 __device__ __forceinline__ void mb_arrive_tx(uint64_t* b, unsigned bytes) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(su32(b)),
                "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mb_arrive(uint64_t* b, int count) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n" ::"r"(su32(b)), "r"(count) : "memory");
 }
 __device__ __forceinline__ bool mb_try_wait(uint64_t* b, unsigned parity) {
   unsigned ok;
@@ -83,11 +86,11 @@ __device__ __forceinline__ bool mb_test_wait(uint64_t* b, unsigned parity) {
 }
 // asynchronous global -> shared copy of `bytes` (8 or 16), the first `src_bytes` of
 // them from src and the rest zero
-__device__ __forceinline__ void cp_async(void* dst, const void* src, int bytes, int src_bytes) {
+__device__ __forceinline__ void cp_async(unsigned dst, const void* src, int bytes, int src_bytes) {
   if (bytes == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(su32(dst)), "l"(src), "r"(src_bytes) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(su32(dst)), "l"(src), "r"(src_bytes) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -97,20 +100,20 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned b
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                ::"r"(su32(dst)), "l"(src), "r"(bytes), "r"(su32(b)) : "memory");
 }
-__device__ __forceinline__ void ch_sync() {   // named barrier 2 among the chain warps
-  asm volatile("bar.sync 2, %0;\n" ::"n"(kSwChain * 32) : "memory");
-}
-__device__ __forceinline__ bool ch_red_or(bool v) {
-  unsigned r;
-  asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 2, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-               : "=r"(r) : "r"((unsigned)v), "n"(kSwChain * 32) : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ bool cw_red_or(bool v) {
+// named barriers of the compute warps: 1 with an OR of a flag, 2 all warps, 3 / 4 the
+// hand-over from one set of warps to the other (the writers arrive, the readers wait)
+__device__ __forceinline__ bool all_red_or(bool v) {
   unsigned r;
   asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
                : "=r"(r) : "r"((unsigned)v), "n"(kSwWarps * 32) : "memory");
   return r != 0;
+}
+__device__ __forceinline__ void all_sync() { asm volatile("bar.sync 2, %0;\n" ::"n"(kSwWarps * 32) : "memory"); }
+__device__ __forceinline__ void hand_sync(unsigned id) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "n"(kSwWarps * 32) : "memory");
+}
+__device__ __forceinline__ void hand_arrive(unsigned id) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "n"(kSwWarps * 32) : "memory");
 }
 
 struct SwArgs {
@@ -119,6 +122,7 @@ struct SwArgs {
   const uint8_t* image;
   float2* x;           // vectors, layout [row][R]
   int64_t R, n;
+  int n0;              // leaf rows
   int64_t col0;        // first column of this launch
   float2* st;          // CTA-private butterfly state: [CTA][state_len][NC]
   int64_t state_len;
@@ -126,32 +130,98 @@ struct SwArgs {
   long long spin_limit;
 };
 
-template <int NC>
-struct Cv {
-  float2 v[NC];
+// ---- shared memory by 32-bit address (every operand of the hot loops lives there)
+typedef unsigned long long f2x;   // two packed FP32 values
+struct f2x2 {
+  f2x a, b;
 };
-
-__device__ __forceinline__ void cmac(float2& acc, const float2 a, const float2 b) {
-  acc.x = fmaf(a.x, b.x, acc.x);
-  acc.x = fmaf(-a.y, b.y, acc.x);
-  acc.y = fmaf(a.x, b.y, acc.y);
-  acc.y = fmaf(a.y, b.x, acc.y);
+__device__ __forceinline__ f2x2 lds_2(unsigned a) {   // 16 bytes: (re, re) and (im, im) of an entry pair
+  f2x2 v;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];\n" : "=l"(v.a), "=l"(v.b) : "r"(a));
+  return v;
 }
+// the same if `on`, else the given value
+__device__ __forceinline__ void lds_2_if(unsigned a, bool on, f2x2& v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %3, 0;\n @p ld.shared.v2.b64 {%0, %1}, [%2];\n}\n"
+               : "+l"(v.a), "+l"(v.b) : "r"(a), "r"((int)on));
+}
+__device__ __forceinline__ float4 lds_f4(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float2 lds_f2(unsigned a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ float lds_f(unsigned a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int2 lds_i2(unsigned a) {
+  int2 v;
+  asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int lds_i(unsigned a) {
+  int v;
+  asm volatile("ld.shared.s32 %0, [%1];\n" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int lds_u16(unsigned a) {
+  int v;
+  asm volatile("ld.shared.u16 %0, [%1];\n" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void lds_i_if(unsigned a, bool on, int& v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %2, 0;\n @p ld.shared.s32 %0, [%1];\n}\n"
+               : "+r"(v) : "r"(a), "r"((int)on));
+}
+__device__ __forceinline__ void sts_f(unsigned a, float v) {
+  asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts_f4(unsigned a, float x, float y, float z, float w) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ f2x ffma2(f2x a, f2x b, f2x c) {   // two FP32 multiply-adds
+  f2x d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f2x fmul2(f2x a, f2x b) {
+  f2x d;
+  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float lo(f2x v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi(f2x v) { return __uint_as_float((unsigned)(v >> 32)); }
 
-// NC consecutive shared-memory entries (16-byte vector load for two columns)
+// Window and slice entries stand in pairs: slots 2i, 2i + 1 of a column as (re, re, im,
+// im), the columns of a pair side by side.  So 16 bytes of coefficients and 16 of inputs
+// give two complex multiply-adds in four packed instructions.
 template <int NC>
-__device__ __forceinline__ Cv<NC> sm_load(const float2* p) {
-  Cv<NC> r;
-  if constexpr (NC == 2) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    r.v[0] = make_float2(v.x, v.y);
-    r.v[1] = make_float2(v.z, v.w);
-  } else {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) r.v[c] = p[c];
+__device__ __forceinline__ unsigned slot_addr(unsigned base, int s) { return base + (s >> 1) * (16 * NC) + (s & 1) * 4; }
+// sums of m v over entry pairs: re re, im im, re im, im re of the even and the odd entries
+struct Acc {
+  f2x rr = 0, ii = 0, ri = 0, ir = 0;
+  __device__ __forceinline__ void set(const f2x2& m, const f2x2& v) {
+    rr = fmul2(m.a, v.a);
+    ii = fmul2(m.b, v.b);
+    ri = fmul2(m.a, v.b);
+    ir = fmul2(m.b, v.a);
   }
-  return r;
-}
+  __device__ __forceinline__ void add(const f2x2& m, const f2x2& v) {
+    rr = ffma2(m.a, v.a, rr);
+    ii = ffma2(m.b, v.b, ii);
+    ri = ffma2(m.a, v.b, ri);
+    ir = ffma2(m.b, v.a, ir);
+  }
+  __device__ __forceinline__ float2 sum() const {
+    return make_float2((lo(rr) + hi(rr)) - (lo(ii) + hi(ii)), (lo(ri) + hi(ri)) + (lo(ir) + hi(ir)));
+  }
+};
 
 // address of a global slot: a vector row (this CTA's columns of x) or a
 // CTA-private state entry
@@ -159,19 +229,21 @@ __device__ __forceinline__ float2* gaddr(const SwArgs& a, int32_t s, float2* xb,
   return s < a.n ? xb + (int64_t)s * a.R : stp + (int64_t)(s - a.n) * nc;
 }
 
-// NC columns of global slot s into dst (shared, 8 * NC bytes) asynchronously; the
+// NC columns of global slot s into shared address dst (8 * NC bytes) asynchronously; the
 // columns beyond this CTA's ncol read as zero.  x rows are 16-byte aligned when the
 // row stride and the CTA's first column are even (vec16).
 template <int NC>
-__device__ __forceinline__ void slot_async(const SwArgs& a, int32_t s, float2* dst, float2* xb, float2* stp, int ncol,
+__device__ __forceinline__ void slot_async(const SwArgs& a, int32_t s, unsigned dst, float2* xb, float2* stp, int ncol,
                                            bool vec16) {
-  if (s < a.n) {
+  if (s < 0) {
+    cp_async(dst, stp, 8 * NC, 0);   // a zero
+  } else if (s < a.n) {
     const float2* src = xb + (int64_t)s * a.R;
     if (NC == 2 && vec16) {
       cp_async(dst, src, 16, 8 * ncol);
     } else {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) cp_async(dst + c, c < ncol ? src + c : src, 8, c < ncol ? 8 : 0);
+      for (int c = 0; c < NC; ++c) cp_async(dst + 8 * c, c < ncol ? src + c : src, 8, c < ncol ? 8 : 0);
     }
   } else {
     const float2* src = stp + (int64_t)(s - a.n) * NC;
@@ -179,410 +251,604 @@ __device__ __forceinline__ void slot_async(const SwArgs& a, int32_t s, float2* d
   }
 }
 
-// One batch in row form, one warp.  Inputs: `in` (the window for resident
-// batches, the warp's gathered slice for global ones); outputs: window slots
-// (RES) or global slots.
-template <int NC, bool RES>
-__device__ void run_rows(const SwArgs& a, const SwDesc& D, const char* bb, const float2* in, float2* win,
-                         float2* xb, float2* stp, int ncol, int lane) {
-  const int32_t* out = reinterpret_cast<const int32_t*>(bb);
-  const int32_t* e0 = reinterpret_cast<const int32_t*>(bb + D.off_e0);
-  const float2* cf = reinterpret_cast<const float2*>(bb + D.off_coef);
-  const int16_t* ix = reinterpret_cast<const int16_t*>(bb + D.off_in);
-  const int glog = D.glog, G = 1 << glog, ng = 32 >> glog;
-  const int q = lane >> glog, l = lane & (G - 1);
-  for (int base = 0; base < D.nrows; base += ng) {
-    const int r = base + q;
-    float2 acc[NC], acc2[NC];
+// ---- one resident tile, one warp.  The coefficients of the lane's first four entry pairs
+// are held in registers, so that they can be fetched before the inputs exist; a longer
+// tile (a multiple of four entries) reads the rest as it goes.  Fewer than four pairs
+// (a phase of very few inputs): the absent ones have coefficient 0 and the lane's first inputs.
+constexpr int kTilePairs = 4;
+constexpr int kPairBytes = 32 * 16;   // one entry pair of all lanes
+template <int NC>
+struct Tile {
+  f2x2 cf[kTilePairs];
+  unsigned va;              // shared address of the lane's first input
+  unsigned coef;            // the lane's entries (shared memory)
+  int np;                   // entry pairs per lane
+  int glog;
+  unsigned dst;             // shared address that this lane stores (a column of) its row's sum to; 0: none
+  bool add;                 // adding to the old value
+};
+// this lane's part of its row's sums
+template <int NC>
+__device__ __forceinline__ void tile_mac(const Tile<NC>& t, float2 (&s)[NC]) {
+  Acc acc[NC];
+  f2x2 v[kTilePairs][NC];
+  const unsigned st = t.np >= kTilePairs ? 16 * NC : 0;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) acc[c] = acc2[c] = make_float2(0.f, 0.f);
-    if (r < D.nrows) {
-      const int ea = e0[r], eb = e0[r + 1];
-      int e = ea + l;
-      // two independent accumulator chains
-      for (; e + G < eb; e += 2 * G) {
-        const float2 m0 = cf[e], m1 = cf[e + G];
-        const Cv<NC> v0 = sm_load<NC>(in + (int)ix[e] * NC);
-        const Cv<NC> v1 = sm_load<NC>(in + (int)ix[e + G] * NC);
+  for (int i = 0; i < kTilePairs; ++i)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          cmac(acc[c], m0, v0.v[c]);
-          cmac(acc2[c], m1, v1.v[c]);
-        }
+    for (int c = 0; c < NC; ++c) v[i][c] = lds_2(t.va + (i == 1 && t.np > 1 ? 16 * NC : i * st) + 16 * c);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) acc[c].set(t.cf[0], v[0][c]);
+#pragma unroll
+  for (int i = 1; i < kTilePairs; ++i)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c].add(t.cf[i], v[i][c]);
+  if (t.np > kTilePairs) {
+    unsigned cp = t.coef + kTilePairs * kPairBytes, vp = t.va + kTilePairs * (16 * NC);
+    int i = kTilePairs;
+#pragma unroll 1
+    for (; i + 1 < t.np; i += 2, cp += 2 * kPairBytes, vp += 2 * (16 * NC)) {
+      f2x2 m[2], w[2][NC];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        m[u] = lds_2(cp + u * kPairBytes);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) w[u][c] = lds_2(vp + u * (16 * NC) + 16 * c);
       }
-      if (e < eb) {
-        const float2 m0 = cf[e];
-        const Cv<NC> v0 = sm_load<NC>(in + (int)ix[e] * NC);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) cmac(acc[c], m0, v0.v[c]);
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c].add(m[u], w[u][c]);
+    }
+    if (i < t.np) {
+      const f2x2 m = lds_2(cp);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c].add(m, lds_2(vp + 16 * c));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) s[c] = acc[c].sum();
+}
+// Sums over a row's 2^glog lanes.  With two columns and more than one lane the first round
+// also parts the columns: the row's first lane keeps column 0, its second column 1 (both in
+// s[0]); with one lane that lane keeps both.
+template <int NC>
+__device__ __forceinline__ void tile_reduce(float2 (&s)[NC], int glog, int lane) {
+  if (glog == 0) return;
+  if constexpr (NC == 2) {
+    const bool odd = lane & 1;
+    const float2 keep = odd ? s[1] : s[0], send = odd ? s[0] : s[1];
+    s[0].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 1);
+    s[0].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 1);
+  } else {
+    s[0].x += __shfl_xor_sync(0xffffffffu, s[0].x, 1);
+    s[0].y += __shfl_xor_sync(0xffffffffu, s[0].y, 1);
+  }
+#pragma unroll
+  for (int g = 1; g < 5; ++g) {
+    if (glog == g) return;
+    s[0].x += __shfl_xor_sync(0xffffffffu, s[0].x, 1 << g);
+    s[0].y += __shfl_xor_sync(0xffffffffu, s[0].y, 1 << g);
+  }
+}
+// whether a lane stores: the row's first NC lanes (its only lane)
+template <int NC>
+__device__ __forceinline__ bool tile_writer(int rows, int glog, int lane) {
+  return (lane >> glog) < rows && (lane & ((1 << glog) - 1)) < NC;
+}
+// a resident tile from the first eight bytes of its descriptor (off | elen, glog, trows)
+template <int NC>
+__device__ __forceinline__ void tile_open(Tile<NC>& t, unsigned gimg, int2 w, unsigned win, int lane) {
+  const unsigned b = gimg + w.x;
+  const int in = lds_u16(b + kSwTileIn + 2 * lane);
+  t.np = (w.y & 0xffff) >> 1;
+  t.glog = (w.y >> 16) & 0xff;
+  const bool wr = tile_writer<NC>(w.y >> 24, t.glog, lane);
+  int o = 0;
+  lds_i_if(b + 4 * (lane >> t.glog), wr, o);
+  t.add = o < 0;
+  t.dst = wr ? slot_addr<NC>(win, o & ~kSwAcc) + (NC == 2 && t.glog > 0 ? 16 * (lane & 1) : 0) : 0;
+  t.coef = b + kSwTileCoef + 16 * lane;
+  t.va = win + in * (8 * NC);
+  if (t.np >= kTilePairs) {
+#pragma unroll
+    for (int i = 0; i < kTilePairs; ++i) t.cf[i] = lds_2(t.coef + i * kPairBytes);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kTilePairs; ++i) {
+      t.cf[i] = f2x2{0, 0};
+      lds_2_if(t.coef + i * kPairBytes, i < t.np && i < 2, t.cf[i]);
+    }
+    // (three pairs: the third by itself)
+    if (t.np == 3) t.cf[2] = lds_2(t.coef + 2 * kPairBytes);
+  }
+}
+// A resident phase's tiles b, b + stride, ... (< nb) of one warp, the first already in `t`.
+template <int NC>
+__device__ __forceinline__ void run_phase(Tile<NC>& t, unsigned gimg, unsigned desc, int b, int nb, int stride, unsigned win,
+                                          int lane) {
+  for (;; b += stride) {
+    const bool more = b + stride < nb;
+    int2 w = make_int2(0, 0);
+    if (more) w = lds_i2(desc + 40 * (b + stride));
+    const int glog = t.glog;
+    const unsigned dst = t.dst;
+    const bool both = NC == 2 && glog == 0;   // the lane stores both columns
+    float2 s[NC], old[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) old[c] = make_float2(0.f, 0.f);
+    if (t.add) {
+      old[0] = make_float2(lds_f(dst), lds_f(dst + 8));
+      if (both) old[NC - 1] = make_float2(lds_f(dst + 16), lds_f(dst + 24));
+    }
+    tile_mac<NC>(t, s);
+    if (more) tile_open<NC>(t, gimg, w, win, lane);
+    tile_reduce<NC>(s, glog, lane);
+    if (dst) {
+      sts_f(dst, old[0].x + s[0].x);
+      sts_f(dst + 8, old[0].y + s[0].y);
+      if (both) {
+        sts_f(dst + 16, old[NC - 1].x + s[NC - 1].x);
+        sts_f(dst + 24, old[NC - 1].y + s[NC - 1].y);
       }
     }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      acc[c].x += acc2[c].x;
-      acc[c].y += acc2[c].y;
-    }
-    // sum over the group's lanes (groups are aligned runs of G lanes)
-    for (int d = G >> 1; d > 0; d >>= 1) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, d);
-        acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, d);
-      }
-    }
-    if (l == 0 && r < D.nrows) {
-      const int32_t o = out[r];
-      const bool add = (o & kSwAcc) != 0;
-      const int32_t s = o & ~kSwAcc;
-      if (RES) {
-        float2* d = win + (int64_t)s * NC;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) d[c] = add ? make_float2(d[c].x + acc[c].x, d[c].y + acc[c].y) : acc[c];
-      } else {
-        float2* d = gaddr(a, s, xb, stp, NC);
-        const int nc = s < a.n ? ncol : NC;
-#pragma unroll
-        for (int c = 0; c < NC; ++c)
-          if (c < nc) {
-            if (add) {
-              const float2 cur = __ldcg(d + c);
-              d[c] = make_float2(cur.x + acc[c].x, cur.y + acc[c].y);
-            } else {
-              d[c] = acc[c];
-            }
-          }
-      }
-    }
+    if (!more) break;
   }
 }
 
-// Sweep-leaf phase: window rows a0 .. a0 + s - 1 replaced by T times them (T the
-// packed triangle), all chain threads (t < nct).  T is stored as a lower
-// triangle, column by column; an upper triangle U is stored reversed (entry
-// (r, c) of the stored triangle is U(s-1-r, s-1-c)), so rev maps the stored
-// rows and columns to window rows s-1-i.  Thread (pair j, column group g) owns
-// stored rows j and s-1-j (s + 1 entries together) and their columns
-// c = g (mod ncg); the lanes of a warp share g and read consecutive entries of
-// one column.  The triangle is not read after the barrier inside.
+// One global batch, one warp: its tiles in turn, inputs from the slice's pairs, old values
+// from its entries as gathered (raw), outputs to global slots.  Few lanes per row, so that
+// the work is mostly the pair loop: one load of coefficients and one of inputs per column
+// for four packed multiply-adds, four pairs in flight.
 template <int NC>
-__device__ void run_tri(const SwDesc& D, bool rev, const float2* T, float2* win, float2* part, int t, int nct) {
-  const int s = D.nrows;
-  float2* b = win + (int64_t)D.a0 * NC;
-  const int npair = s >> 1;
-  int ncg = nct / npair;
-  const int cap = kSwPartBytes / (s * NC * 8);
-  if (ncg > cap) ncg = cap;
-  if (ncg < 1) ncg = 1;
-  if (t < npair * ncg) {
-    const int j = t % npair, g = t / npair;
+__device__ __forceinline__ void run_batch(const SwArgs& a, unsigned desc, unsigned gimg, unsigned pairs, unsigned raw,
+                                          float2* xb, float2* stp, int ncol, bool vec16, int lane) {
+  const int2 w0 = lds_i2(desc), w24 = lds_i2(desc + 24);
+  const unsigned bb = gimg + w0.x, e0 = bb + w24.x, in = bb + lds_i(desc + 32) + 2 * lane;
+  const int nrows = lds_i(desc + 8), old0 = lds_i(desc + 20), glog = (w0.y >> 16) & 0xff, rpt = 32 >> glog;
+  const int nt = (nrows + rpt - 1) >> (5 - glog);
+  const bool one = NC == 2 && glog == 0;               // a lane stores both columns
+  const int c0 = NC == 2 && glog > 0 ? lane & 1 : 0;   // else this one
+  unsigned cp = bb + w24.y + 16 * lane;                // the lane's next coefficients
+  int ea = 0;
+  for (int k = 0; k < nt; ++k) {
+    const int eb = lds_i(e0 + 4 * (k + 1));
+    unsigned vp = pairs + lds_u16(in + 64 * k) * (8 * NC);
+    const bool wr = tile_writer<NC>(nrows - k * rpt, glog, lane);
+    int32_t o = 0;
+    lds_i_if(bb + 4 * (k * rpt + (lane >> glog)), wr, o);
+    Acc acc[NC];
+    int i = (eb - ea) >> 1;
+    ea = eb;
+#pragma unroll 1
+    for (; i >= 4; i -= 4, cp += 4 * kPairBytes, vp += 4 * (16 * NC)) {
+      f2x2 m[4], w[4][NC];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = h == 0 ? j : s - 1 - j;
-      constexpr int U = 4;   // independent accumulator chains
-      float2 acc[4][NC];
+      for (int u = 0; u < 4; ++u) {
+        m[u] = lds_2(cp + u * kPairBytes);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) w[u][c] = lds_2(vp + u * (16 * NC) + 16 * c);
+      }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[u][c] = make_float2(0.f, 0.f);
-      // entry (r, c) at c s - c (c - 1) / 2 + r - c; from c to c + ncg the offset grows by
-      // d = ncg (s - c) - ncg (ncg + 1) / 2, and d shrinks by ncg^2 per step
-      int c = g;
-      int off = c * s - ((c * (c - 1)) >> 1) + r - c;
-      int d = ncg * (s - c) - ((ncg * (ncg + 1)) >> 1);
-      const int dd = ncg * ncg;
-      for (; c + (U - 1) * ncg <= r; c += U * ncg) {
-        float2 m[U];
-        Cv<NC> v[U];
+        for (int c = 0; c < NC; ++c) acc[c].add(m[u], w[u][c]);
+    }
+#pragma unroll 1
+    for (; i > 0; --i, cp += kPairBytes, vp += 16 * NC) {
+      const f2x2 m = lds_2(cp);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          m[u] = T[off];
-          const int cc = c + u * ncg;
-          v[u] = sm_load<NC>(b + (int64_t)(rev ? s - 1 - cc : cc) * NC);
-          off += d;
-          d -= dd;
+      for (int c = 0; c < NC; ++c) acc[c].add(m, lds_2(vp + 16 * c));
+    }
+    float2 s[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) s[c] = acc[c].sum();
+    tile_reduce<NC>(s, glog, lane);
+    if (wr) {
+      float2* d = gaddr(a, o, xb, stp, NC);
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        if ((c == 0 || one) && old0 > 0) {
+          const float2 w = lds_f2(raw + (old0 + k * rpt + (lane >> glog)) * (8 * NC) + 8 * (c0 + c));
+          s[c] = make_float2(w.x + s[c].x, w.y + s[c].y);
         }
+      if (one && (o >= a.n || (vec16 && ncol == 2))) {
+        *reinterpret_cast<float4*>(d) = make_float4(s[0].x, s[0].y, s[NC - 1].x, s[NC - 1].y);
+      } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-          for (int k = 0; k < NC; ++k) cmac(acc[u][k], m[u], v[u].v[k]);
+        for (int c = 0; c < NC; ++c)
+          if ((c == 0 || one) && (c0 + c < ncol || o >= a.n)) d[c0 + c] = s[c];
       }
-      for (; c <= r; c += ncg) {
-        const float2 m = T[off];
-        const Cv<NC> v = sm_load<NC>(b + (int64_t)(rev ? s - 1 - c : c) * NC);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) cmac(acc[0][k], m, v.v[k]);
-        off += d;
-        d -= dd;
-      }
-      const int ro = rev ? s - 1 - r : r;
-#pragma unroll
-      for (int k = 0; k < NC; ++k)
-        part[((int64_t)g * s + ro) * NC + k] =
-            make_float2(acc[0][k].x + acc[1][k].x + acc[2][k].x + acc[3][k].x,
-                        acc[0][k].y + acc[1][k].y + acc[2][k].y + acc[3][k].y);
     }
-  }
-  ch_sync();
-  for (int e = t; e < s * NC; e += nct) {
-    const int r = e / NC, cc = e % NC;
-    float2 sum = make_float2(0.f, 0.f);
-    for (int g = 0; g < ncg; ++g) {
-      const float2 p = part[((int64_t)g * s + r) * NC + cc];
-      sum.x += p.x;
-      sum.y += p.y;
-    }
-    b[(int64_t)r * NC + cc] = sum;
   }
 }
 
+// Sweep-leaf phase: the window rows from slot a0 on replaced by the triangle times them,
+// all compute warps.  A warp's work is four row pairs (stored rows j and s-1-j): lanes =
+// row pair x four column groups x column (two columns) or parity of the step (one).  So
+// every lane has the same 17 steps at order 128, a step's coefficients are consecutive,
+// its inputs four neighbouring column pairs that all row pairs share, and a row's sum
+// needs two shuffle rounds and no other warp; one barrier separates the reads of the rows
+// from their replacement.  Where the run's rows were not all finite, inputs beyond a row's
+// diagonal are masked (0 times a foreign row's Inf would be NaN).  EVEN: the window's slots
+// pair up like the columns (even leaf size).
+template <int NC, bool EVEN>
+__device__ __forceinline__ f2x2 tri_input(unsigned win, int a0, int s, bool up, int p, int c, int n0) {
+  if constexpr (EVEN) {
+    return lds_2(slot_addr<NC>(win, a0 + (up ? s - 2 - 2 * p : 2 * p)) + 16 * c);
+  } else {
+    // columns c0, c0 + 1 by themselves (a column outside the triangle is masked by the caller)
+    const int c0 = up ? s - 2 - 2 * p : 2 * p;
+    unsigned q[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (c0 + u >= 0 && c0 + u < s) {
+        const unsigned d = slot_addr<NC>(win, a0 + sw_row_slot(c0 + u, n0)) + 16 * c;
+        q[u] = __float_as_uint(lds_f(d));
+        q[2 + u] = __float_as_uint(lds_f(d + 8));
+      }
+    f2x2 v;
+    v.a = q[0] | (f2x)q[1] << 32;
+    v.b = q[2] | (f2x)q[3] << 32;
+    return v;
+  }
+}
+// row r's sum over steps [0, n) (r < 0: no such row); coef: the lane's first coefficient
+template <int NC, bool EVEN>
+__device__ __forceinline__ float2 tri_row(int n, unsigned coef, int r, unsigned win, int a0, int s, bool up, int n0, int lane) {
+  const int g = (lane >> 1) & 3, c = NC == 2 ? lane & 1 : 0;
+  // with one column the lane takes every second step
+  const int i0 = NC == 2 ? 0 : lane & 1, di = NC == 2 ? 1 : 2;
+  Acc acc;
+#pragma unroll 1
+  for (int i = i0; i < n; i += di) {
+    const int p = g + 4 * i;
+    const bool in = 2 * p <= r, two = 2 * p < r;   // the pair's first / second stored column within the row
+    f2x2 v{0, 0};
+    if (in) v = tri_input<NC, EVEN>(win, a0, s, up, p, c, n0);
+    const f2x mask = two ? ~0ull : up ? 0xffffffffull << 32 : 0xffffffffull;
+    v.a &= mask;
+    v.b &= mask;
+    acc.add(lds_2(coef + i * 256), v);
+  }
+  return acc.sum();
+}
+// The same for finite inputs of an even leaf size: nothing to mask (the coefficients beyond
+// the diagonal are zero), two steps in flight.  vp: the lane's first input, dv: bytes per step.
 template <int NC>
-// The bound of 512 threads (above the 416 launched) caps the registers at 128 a
-// thread, so that the scheduler that holds four of the 13 warps stays within its
-// 16K registers.
-__global__ void __launch_bounds__(512, 1) k_sweep_cols(SwArgs a) {
+__device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, int dv, int lane) {
+  if (NC == 1) {
+    // every second step per lane
+    cp += (lane & 1) * 256;
+    vp += (lane & 1) * dv;
+    dv *= 2;
+    n = (n + 1 - (lane & 1)) >> 1;
+  }
+  constexpr int cs = NC == 1 ? 512 : 256;
+  Acc acc;
+  int i = 0;
+#pragma unroll 1
+  for (; i + 1 < n; i += 2, cp += 2 * cs, vp += 2 * dv) {
+    const f2x2 m0 = lds_2(cp), v0 = lds_2(vp), m1 = lds_2(cp + cs), v1 = lds_2(vp + dv);
+    acc.add(m0, v0);
+    acc.add(m1, v1);
+  }
+  if (i < n) acc.add(lds_2(cp), lds_2(vp));
+  return acc.sum();
+}
+template <int NC, bool EVEN, bool FAST>
+__device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsigned win, int n0, int warp, int lane) {
+  const int dv = (up ? -64 : 64) * NC;
+  const unsigned vp = slot_addr<NC>(win, a0 + (up ? s - 2 : 0)) + (NC == 2 ? 16 * (lane & 1) : 0) + ((lane >> 1) & 3) * (dv / 4);
+  const int nv = ((s + 1) / 2 + 3) / 4;
+  float val[2] = {0.f, 0.f};
+  unsigned dst[2] = {0, 0};   // 0: nothing to store
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int v = warp + kSwWarps * h;
+    if (v < nv) {
+      const int tw = lds_i(T + 4 * v), n1 = (tw >> 8) & 0xff, nn0 = tw & 0xff;
+      const unsigned coef = T + kSwTriTab + (tw >> 16) * 256 + (lane >> 1) * 16;
+      const int j = 4 * v + (lane >> 3);
+      const int r1 = 2 * j <= s - 1 ? s - 1 - j : -1, r0 = 2 * j < s - 1 ? j : -1;
+      const float2 s1 = FAST ? tri_row_fast<NC>(n1, coef, vp, dv, lane) : tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
+      const float2 s0 = FAST ? tri_row_fast<NC>(nn0, coef + n1 * 256, vp, dv, lane)
+                             : tri_row<NC, EVEN>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
+      // parting the sums over the lanes: a lane pair keeps one row, then one component
+      constexpr int d1 = NC == 2 ? 2 : 1, d2 = 2 * d1;
+      const bool b1 = lane & d1, b2 = lane & d2;
+      float2 keep = b1 ? s0 : s1;
+      const float2 send = b1 ? s1 : s0;
+      keep.x += __shfl_xor_sync(0xffffffffu, send.x, d1);
+      keep.y += __shfl_xor_sync(0xffffffffu, send.y, d1);
+      float w = b2 ? keep.y : keep.x;
+      w += __shfl_xor_sync(0xffffffffu, b2 ? keep.x : keep.y, d2);
+      if (NC == 1) w += __shfl_xor_sync(0xffffffffu, w, 4);
+      const int r = b1 ? r0 : r1;
+      val[h] = w;
+      if (r >= 0 && (NC == 2 || !(lane & 4))) {
+        const int row = up ? s - 1 - r : r;
+        dst[h] = slot_addr<NC>(win, a0 + (EVEN ? row : sw_row_slot(row, n0))) + (NC == 2 ? 16 * (lane & 1) : 0) + (b2 ? 8 : 0);
+      }
+    }
+  }
+  all_sync();
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (dst[h]) sts_f(dst[h], val[h]);
+}
+
+// (out of line: rarely taken)
+template <int NC, bool EVEN>
+__device__ __noinline__ void run_tri_masked(int s, int a0, bool up, unsigned T, unsigned win, int n0, int warp, int lane) {
+  run_tri<NC, EVEN, false>(s, a0, up, T, win, n0, warp, lane);
+}
+
+template <int NC>
+// The bound of 640 threads (above the 544 launched) caps the registers at 96 a thread, so
+// that the scheduler that holds five of the 17 warps stays within its 16K registers.
+__global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
   extern __shared__ __align__(128) char smem[];
-  char* ring = smem;
-  float2* win = reinterpret_cast<float2*>(smem + kSwRingBytes);
-  float2* part = reinterpret_cast<float2*>(smem + kSwRingBytes + kSwWinBytes);
-  __shared__ int s_off[kSwSlots];                 // ring offset of each group in flight
-  __shared__ int s_cnt[kSwSlots];                 // compute warps done with the slot's group
-  __shared__ __align__(8) uint64_t s_mbar[kSwSlots];
-  __shared__ __align__(16) SwGroup s_grec[32];    // the producer's window of group records
+  __shared__ int s_off[kSwFlight];                 // ring offset of each group in flight
+  __shared__ __align__(8) uint64_t s_mbar[kSwFlight];    // group in the slot has arrived
+  __shared__ __align__(8) uint64_t s_free[kSwFlight];    // every compute warp is done with it
   __shared__ int s_abort, s_issued;
+  __shared__ int s_odd;    // the last run (its first group) that loaded a non-finite row
+  const unsigned ring_a = su32(smem), win_a = ring_a + kSwRingBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t lb = a.col0 + (int64_t)blockIdx.x * NC;
   const int ncol = (int)((a.R - lb) < NC ? (a.R - lb) : NC);
   float2* xb = a.x + lb;
   float2* stp = a.st + (int64_t)blockIdx.x * a.state_len * NC;
   if (threadIdx.x == 0) {
-    for (int k = 0; k < kSwSlots; ++k) {
+    for (int k = 0; k < kSwFlight; ++k) {
       mb_init(&s_mbar[k], 1);
-      s_cnt[k] = 0;
+      mb_init(&s_free[k], kSwWarps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     s_abort = 0;
     s_issued = 0;
+    s_odd = -1;
   }
+  // (the unused slots that pad odd input lists are multiplied by zero: no NaN may stand there)
+  for (int e = threadIdx.x; e < kSwWinBytes / 16; e += blockDim.x) sts_f4(win_a + 16 * e, 0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   if (warp == kSwWarps) {
-    // ---- producer: every group of the schedule, in order, into the ring; groups
-    // [oldest, g) are in flight; a group's ring area is free once every compute
-    // warp is done with it, and space is recycled from the oldest group.  Lane 0
-    // keeps the ring state and issues the copies; the warp loads the group
-    // records 32 at a time.
-    int head = 0;
-    int64_t oldest = 0, g = 0;
-    for (; g < a.ngroup; ++g) {
-      if ((g & 31) == 0) {
-        __syncwarp();
-        if (g + lane < a.ngroup) s_grec[lane] = a.groups[g + lane];
-        __syncwarp();
-      }
-      int off = -1;
-      if (lane == 0) {
-        const SwGroup& G = s_grec[g & 31];
-        const int bytes = G.bytes;
-        long long spins = 0;
-        unsigned nap = 32;   // back-off while the ring is full (the compute warps keep the issue slots)
-        for (;;) {
-          while (oldest < g && *(volatile int*)&s_cnt[oldest % kSwSlots] == kSwWarps) ++oldest;
-          __threadfence_block();
-          if (*(volatile int*)&s_abort) break;
-          if (g - oldest < kSwSlots) {
-            if (oldest == g) {
-              off = 0;
-            } else {
-              const int tail = s_off[oldest % kSwSlots];
-              if (head > tail) {
-                if (head + bytes <= kSwRingBytes) off = head;
-                else if (bytes <= tail) off = 0;
-              } else if (head < tail) {
-                if (head + bytes <= tail) off = head;
-              }
+    // ---- producer: every group of the schedule into its place in the ring, one lane each,
+    // 32 groups at a time; a lane may copy once the groups before `need` (its record) are
+    // consumed.  [0, done) are: advanced by looking at 32 slots at once.
+    int done = 0, g0 = 0;
+    const int ngroup = (int)a.ngroup;
+    bool stop = false;
+    for (; g0 < ngroup && !stop; g0 += 32) {
+      const int g = g0 + lane;
+      SwGroup G{0, 0, 0, 0, 0};
+      bool todo = g < ngroup;
+      if (todo) G = a.groups[g];
+      long long spins = 0;
+      for (;;) {
+        const bool go = todo && G.need <= done;
+        if (go) {
+          const int slot = g % kSwFlight;
+          s_off[slot] = G.off;   // published with the arrive (release) below
+          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+          mb_arrive_tx(&s_mbar[slot], (unsigned)G.bytes);
+          bulk_copy(smem + G.off, a.image + G.img, (unsigned)G.bytes, &s_mbar[slot]);
+          todo = false;
+        }
+        const unsigned left = __ballot_sync(0xffffffffu, todo);
+        if (left == 0) break;
+        // groups issued so far: those before the first one left
+        const int issued = g0 + __ffs(left) - 1;
+        const int q = done + lane;
+        const bool free = q < issued && mb_test_wait(&s_free[q % kSwFlight], (unsigned)q / kSwFlight & 1u);
+        const unsigned busy = __ballot_sync(0xffffffffu, !free);
+        const int adv = busy ? __ffs(busy) - 1 : 32;
+        done += adv;
+        if (adv == 0) {
+          if (__any_sync(0xffffffffu, ++spins > a.spin_limit || *(volatile int*)&s_abort)) {
+            if (lane == 0) {
+              atomicExch(&s_abort, 1);
+              s_issued = issued;
             }
-          }
-          if (off >= 0) break;
-          if (++spins > a.spin_limit) {
-            atomicExch(&s_abort, 1);
+            stop = true;
             break;
           }
-          __nanosleep(nap);
-          if (nap < 256) nap <<= 1;
-        }
-        if (off >= 0) {
-          const int slot = (int)(g % kSwSlots);
-          uint64_t* mb = &s_mbar[slot];
-          s_off[slot] = off;
-          s_cnt[slot] = 0;   // published with the arrive (release) below
-          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-          mb_arrive_tx(mb, (unsigned)bytes);
-          bulk_copy(ring + off, a.image + G.img, (unsigned)bytes, mb);
-          head = off + bytes;
+          __nanosleep(20);
         }
       }
-      off = __shfl_sync(0xffffffffu, off, 0);
-      if (off < 0) break;
     }
-    if (lane == 0) s_issued = (int)g;
+    if (!stop && lane == 0) s_issued = ngroup;
     __syncwarp();
   } else {
     const int t = threadIdx.x;
-    const bool chain = warp < kSwChain;
-    float2* slice = win + (int64_t)warp * 2 * kSwGather * NC;   // gather area of global batches (two halves)
+    // gather area of global batches: entries as gathered, then the same in pairs
+    const unsigned raw = win_a + warp * (2 * kSwGather * NC * 8), pairs = raw + kSwGather * NC * 8;
     const bool vec16 = NC == 2 && (a.R % 2) == 0 && (lb % 2) == 0;
-    bool bad = false;   // warp-uniform; after a failed wait the warp only follows the barriers
-    // wait for group g (bounded); returns its image (ring, or global memory after a failure)
-    auto group = [&](int64_t g) -> const char* {
-      const int slot = (int)(g % kSwSlots);
-      if (!bad) {
-        long long spins = 0;
-        bool ok = true;
-        while (!mb_test_wait(&s_mbar[slot], (unsigned)(g / kSwSlots) & 1u)) {
-          if (++spins > a.spin_limit || *(volatile int*)&s_abort) { ok = false; break; }
-          if (spins > 4) __nanosleep(32);   // leave the issue slots to the producer warp
-        }
-        if (__any_sync(0xffffffffu, !ok)) {
-          bad = true;
-          if (lane == 0) atomicExch(&s_abort, 1);
-        }
+    // bounded wait for group g; its image is then at group_at(g)
+    auto wait_group = [&](int g) -> bool {
+      const int slot = g % kSwFlight;
+      const unsigned par = (unsigned)g / kSwFlight & 1u;
+      if (__all_sync(0xffffffffu, mb_test_wait(&s_mbar[slot], par))) return true;
+      long long spins = 1;
+      bool ok = true;
+      while (!mb_test_wait(&s_mbar[slot], par)) {
+        if (++spins > a.spin_limit || *(volatile int*)&s_abort) { ok = false; break; }
+        if (spins > 4) __nanosleep(32);   // leave the issue slots to the producer warp
       }
-      return bad ? reinterpret_cast<const char*>(a.image + a.groups[g].img) : ring + s_off[slot];
+      if (__any_sync(0xffffffffu, !ok)) {
+        if (lane == 0) atomicExch(&s_abort, 1);
+        return false;
+      }
+      return true;
     };
-    int64_t g = 0;
-    while (g < a.ngroup) {
-      const char* gimg = group(g);
-      SwGroupHdr H = *reinterpret_cast<const SwGroupHdr*>(gimg);
-      if (H.flags & SWG_RES) {
-        // ---- a resident run: groups g .. g + H.aux - 1, executed by the chain warps
-        const int64_t g0 = g, gend = g + H.aux;
-        if (!chain) {
-          // the other warps only read the run's length; they release their hold on the
-          // first group's ring area, then wait for the run's end
-          if (!bad) {
-            __syncwarp();
-            if (lane == 0) {
-              __threadfence_block();
-              atomicAdd(&s_cnt[(int)(g % kSwSlots)], 1);
+    auto group_at = [&](int g) -> unsigned { return ring_a + *(volatile int*)&s_off[g % kSwFlight]; };
+    // this warp no longer reads group g's ring area; its owner alone: count kSwWarps
+    auto release = [&](int g, int count) {
+      __syncwarp();
+      if (lane == 0) mb_arrive(&s_free[g % kSwFlight], count);
+    };
+    // Units: resident runs and global phases.  Every unit ends with a barrier of all compute
+    // warps, before which the next unit's first group is waited for; the barrier tells all
+    // warps whether a wait gave up in the unit, and then all stop.
+    const int ngroup = (int)a.ngroup, n0 = a.n0;
+    int g = 0;
+    bool bad = all_red_or(!wait_group(0));   // warp-uniform
+    while (!bad && g < ngroup) {
+      unsigned gimg = group_at(g);
+      int2 H = lds_i2(gimg);                 // nph, flags
+      int off_desc = lds_i(gimg + 24);
+      const int aux = lds_i(gimg + 28);
+      if (!(H.y & SWG_RES)) {
+        // ---- a global phase: groups g .. g + aux - 1, one batch each; this warp's are g + warp,
+        // g + warp + kSwWarps, ...  The gather of its next batch (cp.async) is in flight while the
+        // current one is computed from its regrouped inputs, if that group has arrived -- but for
+        // rows that add, whose old values are still read from the gathered entries.
+        const int gend = g + aux;
+        if (warp > 0) release(g, 1);   // (the first group: its owner, and every warp that read its header)
+        auto gather = [&](unsigned img, unsigned cd) {
+          const int ngl = lds_i(cd + 16);
+          const unsigned gl = img + lds_i(cd) + lds_i(cd + 36);
+          for (int k = lane; k < ngl; k += 32) slot_async<NC>(a, lds_i(gl + 4 * k), raw + k * (8 * NC), xb, stp, ncol, vec16);
+          cp_commit();
+        };
+        auto regroup = [&](int nin) {
+          cp_wait<0>();
+          __syncwarp();
+          for (int k = lane; 2 * k < nin; k += 32) {
+            const unsigned r = raw + k * (16 * NC), p = pairs + k * (16 * NC);
+            const float4 v = lds_f4(r);
+            if constexpr (NC == 2) {
+              const float4 w = lds_f4(r + 16);
+              sts_f4(p, v.x, w.x, v.y, w.y);
+              sts_f4(p + 16, v.z, w.z, v.w, w.w);
+            } else {
+              sts_f4(p, v.x, v.z, v.y, v.w);
             }
           }
-          g = gend;
-          if (cw_red_or(bad)) { bad = true; break; }   // the run is done, its rows written back
-          continue;
-        }
-        const int ct = t, nct = kSwChain * 32;
-        bool stop = false;
-        for (; g < gend && !stop; ++g) {
-          if (g > g0) {
-            gimg = group(g);
-            H = *reinterpret_cast<const SwGroupHdr*>(gimg);
+          __syncwarp();
+        };
+        bool fail = false, ahead = false;   // ahead: the batch's gather has been started
+        for (int q = g + warp; q < gend; q += kSwWarps) {
+          if (!ahead && !(q == g || wait_group(q))) { fail = true; break; }
+          const unsigned img = group_at(q), cd = img + lds_i(img + 24);
+          if (!ahead) gather(img, cd);
+          const int old0 = lds_i(cd + 20);
+          regroup(old0 > 0 ? old0 : lds_i(cd + 16));
+          const int nq = q + kSwWarps;
+          ahead = old0 == 0 && nq < gend &&
+                  __all_sync(0xffffffffu, mb_test_wait(&s_mbar[nq % kSwFlight], (unsigned)nq / kSwFlight & 1u));
+          if (ahead) {
+            const unsigned ni = group_at(nq);
+            gather(ni, ni + lds_i(ni + 24));
           }
-          const int slot = (int)(g % kSwSlots);
-          const SwPhase* tab = reinterpret_cast<const SwPhase*>(gimg + 32);
-          const SwDesc* desc = reinterpret_cast<const SwDesc*>(gimg + H.off_desc);
-          if (H.flags & SWG_BEGIN) {
-            if (!bad) {
-              // the run's rows, all in flight at once
-              for (int r = ct; r < H.beg_hi - H.beg_lo; r += nct) slot_async<NC>(a, H.beg_lo + r, win + r * NC, xb, stp, ncol, vec16);
-              cp_commit();
-              cp_wait<0>();
-            }
-            ch_sync();
-          }
-          int di = 0;
-          bool last_end = false;
-          for (int k = 0; k < H.nph; ++k) {
-            const SwPhase PH = tab[k];
-            last_end = (PH.flags & SWP_END) != 0;
-            if (PH.flags & SWP_TRI) {
-              if (!bad) {
-                const SwDesc D = desc[di];
-                run_tri<NC>(D, (PH.flags & SWP_UPPER) != 0, reinterpret_cast<const float2*>(gimg + D.off), win, part,
-                            ct, nct);
-              } else {
-                ch_sync();   // the barrier inside run_tri
-              }
-            } else if (!bad) {
-              for (int b = warp; b < PH.nb; b += kSwChain) {
-                const SwDesc D = desc[di + b];
-                run_rows<NC, true>(a, D, gimg + D.off, win, win, xb, stp, ncol, lane);
-              }
-            }
-            di += PH.nb;
-            if (PH.flags & SWP_END) {
-              if (ch_red_or(bad)) { bad = true; stop = true; break; }
-            }
-          }
-          if (stop) break;
-          // a group that ends inside a phase (a large phase spread over several groups):
-          // every chain warp must be done with it before it is released
-          if (!last_end) ch_sync();
-          // every chain warp has passed the group's last barrier: the group is consumed
-          // (the run's first group: together with the other warps' holds)
-          if (!bad && ct == 0) {
-            __threadfence_block();
-            if (g == g0) atomicAdd(&s_cnt[slot], kSwChain);
-            else *(volatile int*)&s_cnt[slot] = kSwWarps;
-          }
-          if (H.flags & SWG_ENDRUN) {
-            const int nrow = H.end_hi - H.end_lo;
-            for (int e = ct; e < nrow * NC; e += nct) {
-              const int r = e / NC, c = e % NC;
-              if (c < ncol) xb[(int64_t)(H.end_lo + r) * a.R + c] = win[e];
-            }
-          }
+          run_batch<NC>(a, cd, img, pairs, raw, xb, stp, ncol, vec16, lane);
+          release(q, q == g ? 1 : kSwWarps);
         }
         g = gend;
-        if (cw_red_or(bad)) { bad = true; break; }   // the run is done, its rows written back
+        // (the barrier also makes every compute warp's writes visible to the next phase)
+        bad = all_red_or(fail || (g < ngroup && !wait_group(g)));
         continue;
       }
-      // ---- a part of a global phase: batches round-robin over all compute warps
-      {
-        const int slot = (int)(g % kSwSlots);
-        const SwPhase PH = *reinterpret_cast<const SwPhase*>(gimg + 32);
-        const SwDesc* desc = reinterpret_cast<const SwDesc*>(gimg + H.off_desc);
-        if (!bad) {
-          // this warp's batches b0, b0 + 12, ...: the gather of the next one (cp.async into
-          // the other half of the warp's slice) is in flight while this one is computed
-          const int b0 = (warp - H.aux + kSwWarps) % kSwWarps;
-          auto gather = [&](int b, float2* dst) {
-            const SwDesc& D = desc[b];
-            const int32_t* gl = reinterpret_cast<const int32_t*>(gimg + D.off + D.off_gl);
-            for (int k = lane; k < D.ngl; k += 32) slot_async<NC>(a, gl[k], dst + k * NC, xb, stp, ncol, vec16);
-            cp_commit();
-          };
-          int buf = 0;
-          if (b0 < PH.nb) gather(b0, slice);
-          for (int b = b0; b < PH.nb; b += kSwWarps) {
-            const int bn = b + kSwWarps;
-            if (bn < PH.nb) {
-              gather(bn, slice + (buf ^ 1) * kSwGather * NC);
-              cp_wait<1>();
-            } else {
-              cp_wait<0>();
-            }
-            __syncwarp();
-            const SwDesc D = desc[b];
-            run_rows<NC, false>(a, D, gimg + D.off, slice + buf * kSwGather * NC, win, xb, stp, ncol, lane);
-            __syncwarp();
-            buf ^= 1;
-          }
+      // ---- a resident run: groups g .. g + aux - 1
+      const int gend = g + aux, unit = g;
+      const int2 rows = lds_i2(gimg + 8);   // the run's rows [lo, hi)
+#pragma unroll 4
+      for (int r = t; r < rows.y - rows.x; r += kSwWarps * 32) {
+        const float2* src = xb + (int64_t)(rows.x + r) * a.R;
+        const unsigned d = slot_addr<NC>(win_a, sw_row_slot(r, n0));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const float2 v = c < ncol ? __ldcg(src + c) : make_float2(0.f, 0.f);
+          if (!isfinite(v.x) || !isfinite(v.y)) *(volatile int*)&s_odd = unit;
+          sts_f(d + 16 * c, v.x);
+          sts_f(d + 16 * c + 8, v.y);
         }
-        if (PH.flags & SWP_END) {
-          // end of the phase: every compute warp's writes are visible to the next phase
-          if (cw_red_or(bad)) { bad = true; break; }
-          if (t == 0) {
-            __threadfence_block();
-            *(volatile int*)&s_cnt[slot] = kSwWarps;
-          }
-        } else if (!bad) {
-          __syncwarp();
-          if (lane == 0) {
-            __threadfence_block();
-            atomicAdd(&s_cnt[slot], 1);   // this warp no longer reads the group's ring area
-          }
-        }
-        ++g;
       }
+      const int set = warp >= kSwSet ? SWP_SET1 : 0, wset = warp & (kSwSet - 1);
+      bool hand = false, sync = true;   // the previous phase hands over to this one's set / all warps meet
+      unsigned hid = 3;       // barrier of the next hand-over (3 and 4 in turn)
+      int2 P0 = lds_i2(gimg + 32), nH = H, nP = H;   // the group's first phase; the next group's header
+      unsigned nimg = 0;                             // the next group's image once seen, else 0
+      int noff = 0;
+      while (g < gend) {
+        for (int k = 0; k < H.x; ++k) {
+          int2 PH;   // nb, flags
+          if (!bad) {
+            PH = k == 0 ? P0 : lds_i2(gimg + 32 + 8 * k);
+            // the group's last phase: look whether the next group has arrived, and read its header
+            if (k + 1 == H.x && g + 1 < gend &&
+                __all_sync(0xffffffffu, mb_test_wait(&s_mbar[(g + 1) % kSwFlight], (unsigned)(g + 1) / kSwFlight & 1u))) {
+              nimg = group_at(g + 1);
+              nH = lds_i2(nimg);
+              noff = lds_i(nimg + 24);
+              nP = lds_i2(nimg + 32);
+            }
+          } else {
+            // after a wait that gave up: follow the run's barriers from the schedule in global memory
+            const SwPhase p = reinterpret_cast<const SwPhase*>(a.image + a.groups[g].img + 32)[k];
+            PH = make_int2(p.nb, p.flags);
+          }
+          const bool all = (PH.y & SWP_ALL) != 0, tri = (PH.y & SWP_TRI) != 0;
+          const bool mine = all || (PH.y & SWP_SET1) == set;
+          const int first = all ? (warp - (PH.y >> kSwPhaseWarp)) & (kSwWarps - 1) : wset;
+          const bool rowsp = mine && !tri && !bad && first < PH.x;
+          const unsigned desc = gimg + off_desc + 40 * ((PH.y >> kSwPhaseBase) & kSwBaseMask);
+          Tile<NC> tile;
+          if (rowsp) tile_open<NC>(tile, gimg, lds_i2(desc + 40 * first), win_a, lane);   // nothing here depends on the inputs
+          if (hand) {
+            if (mine) hand_sync(hid);
+            hid ^= 7;
+          } else if (sync) {
+            all_sync();
+          }
+          if (rowsp) {
+            run_phase<NC>(tile, gimg, desc, first, PH.x, all ? kSwWarps : kSwSet, win_a, lane);
+          } else if (tri) {
+            if (!bad) {
+              const int toff = lds_i(desc), s = lds_i(desc + 8), a0 = lds_i(desc + 20);
+              const bool up = (PH.y & SWP_UPPER) != 0;
+              if (n0 & 1) run_tri_masked<NC, false>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+              else if (*(volatile int*)&s_odd == unit) run_tri_masked<NC, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+              else run_tri<NC, true, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+            } else {
+              all_sync();   // the barrier inside the triangle product
+            }
+          }
+          hand = (PH.y & SWP_HAND) != 0;
+          sync = (PH.y & SWP_END) != 0;   // (a phase's parts need no barrier between them)
+          if (hand && mine) hand_arrive(hid);
+        }
+        if (!bad) release(g, 1);
+        if (++g < gend) {
+          if (!bad && nimg == 0) {
+            bad = !wait_group(g);
+            if (!bad) {
+              nimg = group_at(g);
+              nH = lds_i2(nimg);
+              noff = lds_i(nimg + 24);
+              nP = lds_i2(nimg + 32);
+            }
+          }
+          if (!bad) {
+            gimg = nimg;
+            H = nH;
+            off_desc = noff;
+            P0 = nP;
+            nimg = 0;
+          } else {
+            H.x = reinterpret_cast<const SwGroupHdr*>(a.image + a.groups[g].img)->nph;
+          }
+        }
+      }
+      all_sync();   // the run's last phase is done
+      if (!bad)
+        for (int e = t; e < (rows.y - rows.x) * NC; e += kSwWarps * 32) {
+          const int r = e / NC, c = e % NC;
+          const unsigned d = slot_addr<NC>(win_a, sw_row_slot(r, n0)) + 16 * c;
+          if (c < ncol) xb[(int64_t)(rows.x + r) * a.R + c] = make_float2(lds_f(d), lds_f(d + 8));
+        }
+      bad = all_red_or(bad || (g < ngroup && !wait_group(g)));   // (the rows are written back)
     }
     if (bad && t == 0) {
       atomicExch(&s_abort, 1);
@@ -594,16 +860,19 @@ __global__ void __launch_bounds__(512, 1) k_sweep_cols(SwArgs a) {
     // give the copies still in flight a second bounded wait before leaving
     const int iss = s_issued;
     for (int q = 0; q < iss; ++q) {
-      if (q + kSwSlots < iss) continue;
+      if (q + kSwFlight < iss) continue;
       long long spins = 0;
-      while (!mb_try_wait(&s_mbar[q % kSwSlots], (unsigned)(q / kSwSlots) & 1u) &&
+      while (!mb_try_wait(&s_mbar[q % kSwFlight], (unsigned)(q / kSwFlight) & 1u) &&
              ++spins < drain_limit(a.spin_limit)) {
       }
     }
   }
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int k = 0; k < kSwSlots; ++k) mb_inval(&s_mbar[k]);
+    for (int k = 0; k < kSwFlight; ++k) {
+      mb_inval(&s_mbar[k]);
+      mb_inval(&s_free[k]);
+    }
 }
 
 template <int NC>
@@ -625,6 +894,7 @@ int launch_nc(const DevFactor& df, const DevSched& sc, float2* vec, int64_t R, i
   a.x = vec;
   a.R = R;
   a.n = df.n;
+  a.n0 = (int)df.n0;
   a.col0 = col0;
   a.st = st;
   a.state_len = df.state_len;
