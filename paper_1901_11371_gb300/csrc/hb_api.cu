@@ -783,9 +783,9 @@ int hb_apply(hb_factor_t f, int op, const void* x, void* y, int64_t nrhs, int64_
   void* xi = f->ws.get(WS_VEC0, bytes);
   void* yi = f->ws.get(WS_VEC1, bytes);
   if (!xi || !yi) { set_error("hb_apply: workspace allocation failed"); return HB_ENOMEM; }
-  if ((rc = launch_gather_cols(x, vt, ld, df.n, nrhs, xi, vt, 1.0, st))) return rc;
+  if ((rc = launch_gather_cols(x, vt, ld, df.n, nrhs, xi, 1.0, st))) return rc;
   if ((rc = apply_internal(f, p, op == HB_OP_H, xi, yi, nrhs, st))) return rc;
-  return launch_scatter_cols(yi, vt, df.n, nrhs, y, vt, ld, 1.0, st);
+  return launch_scatter_cols(yi, vt, df.n, nrhs, y, ld, st);
 }
 
 int hb_apply_adjoint(hb_factor_t f, const void* x, void* y, int64_t nrhs, int64_t ld, void* stream) {
@@ -811,11 +811,11 @@ static int sweeps(hb_factor_t f, int op, const void* b, void* x, int64_t nrhs, i
   } else {
     v = f->ws.get(WS_VEC0, (size_t)df.n * nrhs * vt_size(vt));
     if (!v) { set_error("%s: workspace allocation failed", who); return HB_ENOMEM; }
-    if ((rc = launch_gather_cols(b, vt, ld, df.n, nrhs, v, vt, 1.0, st))) return rc;
+    if ((rc = launch_gather_cols(b, vt, ld, df.n, nrhs, v, 1.0, st))) return rc;
   }
   if (first >= 0 && (rc = sweep_internal(f, p, first, v, nrhs, st))) return rc;
   if (second >= 0 && (rc = sweep_internal(f, p, second, v, nrhs, st))) return rc;
-  if (nrhs > 1) return launch_scatter_cols(v, vt, df.n, nrhs, x, vt, ld, 1.0, st);
+  if (nrhs > 1) return launch_scatter_cols(v, vt, df.n, nrhs, x, ld, st);
   return HB_OK;
 }
 
@@ -842,7 +842,7 @@ int hb_residual(hb_factor_t f, int op, const void* b, const void* x, void* r, in
   void* xi = f->ws.get(WS_VEC0, bytes);
   void* yi = f->ws.get(WS_VEC1, bytes);
   if (!xi || !yi) { set_error("hb_residual: workspace allocation failed"); return HB_ENOMEM; }
-  if ((rc = launch_gather_cols(x, 0, ld, df.n, nrhs, xi, 0, 1.0, st))) return rc;
+  if ((rc = launch_gather_cols(x, 0, ld, df.n, nrhs, xi, 1.0, st))) return rc;
   if ((rc = apply_internal(f, p, op == HB_OP_H, xi, yi, nrhs, st))) return rc;
   return launch_residual_cols(b, ld, yi, df.n, nrhs, r, st);
 }

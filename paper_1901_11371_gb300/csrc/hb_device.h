@@ -159,12 +159,9 @@ int set_grid_min(DevFactor& df, const PackedHost& ph, int grid_min, cudaStream_t
 // `cols` columns per CTA.
 int build_candidates(DevFactor& df, const PackedHost& ph, int cls, int64_t cols, cudaStream_t st);
 
-// Layout conversion between the ABI's column-major [R][ld] blocks and the
-// internal [row][R] layout, with optional precision change and scaling.
-// src_t / dst_t: 0 = double2, 1 = float2.
-int launch_gather_cols(const void* src, int src_t, int64_t ld, int64_t n, int64_t R, void* dst, int dst_t,
-                       double scale, cudaStream_t st);
-int launch_scatter_cols(const void* src, int src_t, int64_t n, int64_t R, void* dst, int dst_t, int64_t ld,
-                        double scale, cudaStream_t st);
+// Layout conversion between the ABI's column-major [R][ld] blocks and the internal
+// [row][R] layout; the gather can scale.  type 0: double2, 1: float2.
+int launch_gather_cols(const void* src, int type, int64_t ld, int64_t n, int64_t R, void* dst, double scale, cudaStream_t st);
+int launch_scatter_cols(const void* src, int type, int64_t n, int64_t R, void* dst, int64_t ld, cudaStream_t st);
 
 }  // namespace hb

@@ -99,7 +99,7 @@ extern "C" int hb_apply_noalloc(hb_factor_t f, int op, const void* x, void* y, i
   if (nrhs == 1) return launch_apply(df, p, op == HB_OP_H, x, y, 1, state, st);
   void* xi = s + state_bytes;
   void* yi = s + state_bytes + vec_bytes;
-  if ((rc = launch_gather_cols(x, vt, ld, df.n, nrhs, xi, vt, 1.0, st))) return rc;
+  if ((rc = launch_gather_cols(x, vt, ld, df.n, nrhs, xi, 1.0, st))) return rc;
   if ((rc = launch_apply(df, p, op == HB_OP_H, xi, yi, nrhs, state, st))) return rc;
-  return launch_scatter_cols(yi, vt, df.n, nrhs, y, vt, ld, 1.0, st);
+  return launch_scatter_cols(yi, vt, df.n, nrhs, y, ld, st);
 }

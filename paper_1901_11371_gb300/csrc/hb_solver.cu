@@ -259,28 +259,12 @@ __global__ void k_nonfinite(const double2* __restrict__ a, int64_t ld, int64_t n
   }
 }
 
-// r(col-major) = b(col-major) - y([row][R])
-__global__ void k_residual_cols(const double2* __restrict__ b, int64_t ld, const double2* __restrict__ y, int64_t n,
-                                int64_t R, double2* __restrict__ r) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (; e < n * R; e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t row = e / R, c = e % R;
-    double2 bb = b[c * ld + row], yy = y[e];
-    r[c * ld + row] = {bb.x - yy.x, bb.y - yy.y};
-  }
-}
-
 // max that keeps a NaN once seen (reports of diverged columns)
 static inline double nan_max(double a, double b) { return (std::isnan(a) || std::isnan(b)) ? NAN : std::max(a, b); }
 
 static inline int gsz(int64_t total) {
   int64_t g = (total + 255) / 256;
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 16));
-}
-
-int launch_residual_cols(const void* b, int64_t ld, const void* y, int64_t n, int64_t R, void* r, cudaStream_t st) {
-  k_residual_cols<<<gsz(n * R), 256, 0, st>>>((const double2*)b, ld, (const double2*)y, n, R, (double2*)r);
-  return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
 }
 
 // ---------------------------------------------------------------------------
@@ -775,7 +759,7 @@ extern "C" int hb_gmres(hb_factor_t f, int op, const void* b_phys, void* x, int6
   if (cudaStreamSynchronize(st) != cudaSuccess) { set_error("hb_gmres: CUDA error"); return HB_ECUDA; }
   if (hflag) { set_error("hb_gmres: right-hand side contains NaN/Inf"); return HB_ENAN; }
 
-  if ((rc = launch_gather_cols(b_phys, 0, ld, n, R, bh, 0, df.scale, st))) return rc;
+  if ((rc = launch_gather_cols(b_phys, 0, ld, n, R, bh, df.scale, st))) return rc;
   cudaMemsetAsync(xv, 0, vbytes, st);
   std::vector<double> bnorm;
   if ((rc = norms(d, bh, bnorm))) return rc;
@@ -1174,9 +1158,9 @@ extern "C" int hb_gmres(hb_factor_t f, int op, const void* b_phys, void* x, int6
   if (!mixed) {
     cudaMemcpyAsync(tmp2, xv, vbytes, cudaMemcpyDeviceToDevice, st);
     if ((rc = sweep_internal(f, PREC_F64, up, tmp2, R, st))) return rc;
-    if ((rc = launch_scatter_cols(tmp2, 0, n, R, x, 0, ld, 1.0, st))) return rc;
+    if ((rc = launch_scatter_cols(tmp2, 0, n, R, x, ld, st))) return rc;
   } else {
-    if ((rc = launch_scatter_cols(xv, 0, n, R, x, 0, ld, 1.0, st))) return rc;
+    if ((rc = launch_scatter_cols(xv, 0, n, R, x, ld, st))) return rc;
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) { set_error("hb_gmres: CUDA error"); return HB_ECUDA; }
   if ((rc = hb_status(f, stream))) return rc;   // the last sweep's bounded waits
@@ -1278,13 +1262,13 @@ extern "C" int hb_tfqmr(hb_factor_t f, int op, const void* b_phys, const void* r
     cudaMemcpyAsync(dst, c.data(), R * sizeof(double2), cudaMemcpyHostToDevice, st);
     return dst;
   };
-  if ((rc = launch_gather_cols(b_phys, 0, ld, n, R, bh, 0, df.scale, st))) return rc;
+  if ((rc = launch_gather_cols(b_phys, 0, ld, n, R, bh, df.scale, st))) return rc;
   std::vector<double> bnorm, tau;
   if ((rc = norms(d, bh, bnorm))) return rc;
   cudaMemcpyAsync(w, bh, vbytes, cudaMemcpyDeviceToDevice, st);
   if ((rc = sweep_internal(f, px, lo, w, R, st))) return rc;
   cudaMemcpyAsync(u, w, vbytes, cudaMemcpyDeviceToDevice, st);
-  if (rstar) { if ((rc = launch_gather_cols(rstar, 0, ld, n, R, rs, 0, 1.0, st))) return rc; }
+  if (rstar) { if ((rc = launch_gather_cols(rstar, 0, ld, n, R, rs, 1.0, st))) return rc; }
   else cudaMemcpyAsync(rs, w, vbytes, cudaMemcpyDeviceToDevice, st);
   cudaMemsetAsync(y, 0, vbytes, st);
   cudaMemsetAsync(dd, 0, vbytes, st);
@@ -1382,7 +1366,7 @@ extern "C" int hb_tfqmr(hb_factor_t f, int op, const void* b_phys, const void* r
   }
   // report the final true residual of every column, return x = U'^{-1} y
   if ((rc = true_residual())) return rc;
-  if ((rc = launch_scatter_cols(t2, 0, n, R, x, 0, ld, 1.0, st))) return rc;
+  if ((rc = launch_scatter_cols(t2, 0, n, R, x, ld, st))) return rc;
   if (cudaStreamSynchronize(st) != cudaSuccess) { set_error("hb_tfqmr: CUDA error"); return HB_ECUDA; }
   if ((rc = hb_status(f, stream))) return rc;   // the last sweep's bounded waits
   int nconv = 0, nbroken = 0;
