@@ -37,8 +37,56 @@ using zc = std::complex<double>;
 // ---------------------------------------------------------------------------
 // BLAS-1 style kernels on [row][R] blocks (double2)
 // ---------------------------------------------------------------------------
-static constexpr int kRedBlocks = 304;   // 2 x 152 SMs
+static constexpr int kRedBlocks = 304;   // 2 x 152 SMs; most row blocks of a dot product
 static constexpr int kRedThreads = 256;
+// Row blocks of a dot product over n rows of R columns: four rows a thread (FP32 vectors: one,
+// for their per-thread sums are FP32), so that a short vector is not spread over blocks that
+// hold little but their own reduction, and at most kRedBlocks.  (1,024 rows, one FP64 column, 25 vectors: 304 blocks whose first thread summed
+// 256 values in turn and a final sum of 304 took 68 + 32 us; one block per vector takes 7 + 4.)
+template <class VT>
+static inline int red_blocks(int64_t n, int64_t R) {
+  const int64_t per = (sizeof(VT) == sizeof(double2) ? 4 : 1) * (R >= kRedThreads ? 1 : kRedThreads / R);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (n + per - 1) / per));
+}
+// Columns a CTA of the final sums takes (a power of two); the other threads share the blocks.
+static inline int fin_cols(int64_t R) {
+  int c = 1;
+  while (c < R && c < 32) c *= 2;
+  return c;
+}
+static inline dim3 fin_grid(int64_t R, int nvec) {
+  return dim3((unsigned)((R + fin_cols(R) - 1) / fin_cols(R)), (unsigned)nvec);
+}
+// Sum over the row blocks of partial[blk][r], r = blockIdx.x rc + threadIdx.x % rc, in an order
+// that nblk and rc fix.  Latency-bound: 256 / rc threads share a column's loads and join over
+// a tree (one thread a column in a chain of 304 loads: 25 - 47 us; so: 4).  Whole CTA; the
+// sum is valid in the threads below rc.
+__device__ __forceinline__ double2 block_sums(const double2* __restrict__ partial, int nblk, int64_t R, int rc) {
+  __shared__ double2 red[kRedThreads];
+  const int t = threadIdx.x, slice = t / rc, S = kRedThreads / rc;
+  const int64_t r = (int64_t)blockIdx.x * rc + t % rc;
+  double2 s = {0.0, 0.0};
+  if (r < R) {
+#pragma unroll 4
+    for (int b = slice; b < nblk; b += S) {
+      const double2 p = partial[(int64_t)b * R + r];
+      s.x += p.x;
+      s.y += p.y;
+    }
+  }
+  red[t] = s;
+  __syncthreads();
+  for (int off = S / 2; off > 0; off >>= 1) {
+    if (slice < off) {
+      const double2 o = red[t + off * rc];
+      s.x += o.x;
+      s.y += o.y;
+      red[t] = s;
+    }
+    __syncthreads();
+  }
+  return s;
+}
 
 // partial[v][blk][r] = sum over this block's rows of conj(V_v[row][r]) * w[row][r]
 // (VT = double2: FP64 arithmetic; VT = float2: FP32 products and per-thread
@@ -59,39 +107,40 @@ __global__ void k_dots_partial(const VT* __restrict__ V, int64_t vstride, int nv
     int g = (R >= kRedThreads) ? 0 : t / (int)R;
     S ax = 0, ay = 0;
     if (g < G && r < R) {
+#pragma unroll 4
       for (int64_t row = row0 + g; row < row1; row += G) {
         VT a = Vv[row * R + r], b = w[row * R + r];
         ax = fma(a.x, b.x, fma(a.y, b.y, ax));
         ay = fma(a.x, b.y, fma(-a.y, b.x, ay));
       }
     }
+    if (R >= kRedThreads) {
+      if (r < R) partial[((int64_t)v * gridDim.x + blockIdx.x) * R + r] = double2{(double)ax, (double)ay};
+      continue;
+    }
     red[t] = double2{(double)ax, (double)ay};
     __syncthreads();
-    if (R >= kRedThreads) {
-      if (r < R) partial[((int64_t)v * gridDim.x + blockIdx.x) * R + r] = red[t];
-    } else if (t < R) {
-      double2 s = {0.0, 0.0};
-      for (int gg = 0; gg < G; ++gg) { s.x += red[gg * R + t].x; s.y += red[gg * R + t].y; }
-      partial[((int64_t)v * gridDim.x + blockIdx.x) * R + t] = s;
+    int off = 1;
+    while (2 * off < G) off *= 2;
+    for (; off > 0; off >>= 1) {
+      if (g < off && g + off < G) {
+        const double2 o = red[t + off * (int)R];
+        red[t].x += o.x;
+        red[t].y += o.y;
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    if (R < kRedThreads) break;
+    if (t < R) partial[((int64_t)v * gridDim.x + blockIdx.x) * R + t] = red[t];
+    break;
   }
 }
 
-// out[v][r] = sum_blk partial[v][blk][r] (fixed order)
-__global__ void k_dots_final(const double2* __restrict__ partial, int nblk, int nvec, int64_t R, double2* out) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)nvec * R) return;
-  int v = (int)(e / R);
-  int64_t r = e % R;
-  double2 s = {0.0, 0.0};
-  for (int b = 0; b < nblk; ++b) {
-    double2 p = partial[((int64_t)v * nblk + b) * R + r];
-    s.x += p.x;
-    s.y += p.y;
-  }
-  out[e] = s;
+// out[v][r] = sum_blk partial[v][blk][r]
+__global__ void __launch_bounds__(kRedThreads) k_dots_final(const double2* __restrict__ partial, int nblk, int64_t R,
+                                                            int rc, double2* out) {
+  const double2 s = block_sums(partial + (int64_t)blockIdx.y * nblk * R, nblk, R, rc);
+  const int64_t r = (int64_t)blockIdx.x * rc + threadIdx.x;
+  if (threadIdx.x < rc && r < R) out[(int64_t)blockIdx.y * R + r] = s;
 }
 
 // w[row][r] -= sum_v V_v[row][r] h[v][r]   (h and the arithmetic in the precision of VT)
@@ -167,7 +216,7 @@ template <class VT>
 static void launch_sub_dots(const VT* V, int64_t vstride, int nvec, const VT* h, VT* w, int64_t n, int64_t R,
                             double2* partial, cudaStream_t s) {
   if constexpr (sizeof(VT) == 8) {
-    const dim3 grid(kRedBlocks, (unsigned)((R + kRedThreads - 1) / kRedThreads));
+    const dim3 grid(red_blocks<VT>(n, R), (unsigned)((R + kRedThreads - 1) / kRedThreads));
     if (nvec <= 8) k_sub_dots<VT, 8><<<grid, kRedThreads, 0, s>>>(V, vstride, nvec, h, w, n, R, partial);
     else if (nvec <= 16) k_sub_dots<VT, 16><<<grid, kRedThreads, 0, s>>>(V, vstride, nvec, h, w, n, R, partial);
     else k_sub_dots<VT, 32><<<grid, kRedThreads, 0, s>>>(V, vstride, nvec, h, w, n, R, partial);
@@ -354,9 +403,9 @@ struct Dev {
 };
 
 // the partial dot products in d.red_partial reduced to hh[v*R + r] (host copy)
-static int dots_finish(Dev& d, int nvec, std::vector<zc>& hh) {
+static int dots_finish(Dev& d, int nblk, int nvec, std::vector<zc>& hh) {
   int64_t tot = (int64_t)nvec * d.R;
-  k_dots_final<<<(unsigned)((tot + 255) / 256), 256, 0, d.st>>>(d.red_partial, kRedBlocks, nvec, d.R, d.red_out); count_launch(d.f, 1);
+  k_dots_final<<<fin_grid(d.R, nvec), kRedThreads, 0, d.st>>>(d.red_partial, nblk, d.R, fin_cols(d.R), d.red_out); count_launch(d.f, 1);
   hh.resize(tot);
   if (cudaMemcpyAsync(hh.data(), d.red_out, tot * sizeof(double2), cudaMemcpyDeviceToHost, d.st) != cudaSuccess)
     return HB_ECUDA;
@@ -377,9 +426,9 @@ static int dots_finish(Dev& d, int nvec, std::vector<zc>& hh) {
 // h[v][r] = <V_v, w>_r for v < nvec (host copy returned in hh[v*R + r])
 template <class VT>
 static int dots(Dev& d, const VT* V, int64_t vstride, int nvec, const VT* w, std::vector<zc>& hh) {
-  dim3 grid(kRedBlocks, nvec);
+  dim3 grid(red_blocks<VT>(d.n, d.R), nvec);
   k_dots_partial<VT><<<grid, kRedThreads, 0, d.st>>>(V, vstride, nvec, w, d.n, d.R, d.red_partial); count_launch(d.f, 1);
-  return dots_finish(d, nvec, hh);
+  return dots_finish(d, (int)grid.x, nvec, hh);
 }
 
 // CGS2: orthogonalise w against V_0..V_{nvec-1}; returns h (nvec x R) and ||w|| (R).
@@ -394,7 +443,7 @@ static int cgs2(Dev& d, const VT* V, int64_t vstride, int nvec, VT* w, std::vect
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 0 || !fused) {
       if ((rc = dots(d, V, vstride, nvec, w, pass ? h2 : h1))) return rc;
-    } else if ((rc = dots_finish(d, nvec, h2))) {
+    } else if ((rc = dots_finish(d, red_blocks<VT>(d.n, d.R), nvec, h2))) {
       return rc;
     }
     std::vector<zc>& hp = pass ? h2 : h1;
@@ -520,15 +569,10 @@ __device__ __forceinline__ double2 z_cmul(double2 a, double2 b) {   // conj(a) b
 
 // beta = ||r|| per column (the fixed-order sum of the partial dot products),
 // 1 / beta for the start vector, g = beta e_1, the column's target and state
-__global__ void k_cyc_start(const double2* __restrict__ partial, int nblk, Cyc c) {
-  const int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= c.R) return;
-  double2 sum = {0.0, 0.0};
-  for (int b = 0; b < nblk; ++b) {
-    const double2 p = partial[(int64_t)b * c.R + col];
-    sum.x += p.x;
-    sum.y += p.y;
-  }
+__global__ void __launch_bounds__(kRedThreads) k_cyc_start(const double2* __restrict__ partial, int nblk, int rc, Cyc c) {
+  const double2 sum = block_sums(partial, nblk, c.R, rc);
+  const int64_t col = (int64_t)blockIdx.x * rc + threadIdx.x;
+  if (threadIdx.x >= rc || col >= c.R) return;
   const double beta = sqrt(fmax(sum.x, 0.0));
   c.inv[col] = beta > 0 ? 1.0 / beta : 1.0;
   c.g[col * (c.m + 1)] = {beta, 0.0};
@@ -538,17 +582,12 @@ __global__ void k_cyc_start(const double2* __restrict__ partial, int nblk, Cyc c
 
 // one CGS2 pass's coefficients: hacc (+)= <V_v, w>, cvec = the same in the basis precision
 template <class VT>
-__global__ void k_cgs_final(const double2* __restrict__ partial, int nblk, int nvec, Cyc c, int pass) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)nvec * c.R) return;
-  const int v = (int)(e / c.R);
-  const int64_t r = e % c.R;
-  double2 sum = {0.0, 0.0};
-  for (int b = 0; b < nblk; ++b) {
-    const double2 p = partial[((int64_t)v * nblk + b) * c.R + r];
-    sum.x += p.x;
-    sum.y += p.y;
-  }
+__global__ void __launch_bounds__(kRedThreads) k_cgs_final(const double2* __restrict__ partial, int nblk, int rc, Cyc c,
+                                                           int pass) {
+  const double2 sum = block_sums(partial + (int64_t)blockIdx.y * nblk * c.R, nblk, c.R, rc);
+  const int64_t r = (int64_t)blockIdx.x * rc + threadIdx.x;
+  if (threadIdx.x >= rc || r >= c.R) return;
+  const int64_t e = (int64_t)blockIdx.y * c.R + r;
   double2 h = sum;
   if (pass) h = {c.hacc[e].x + sum.x, c.hacc[e].y + sum.y};
   c.hacc[e] = h;
@@ -556,15 +595,10 @@ __global__ void k_cgs_final(const double2* __restrict__ partial, int nblk, int n
 }
 
 // ||w|| and 1 / ||w|| per column
-__global__ void k_norm_final(const double2* __restrict__ partial, int nblk, Cyc c) {
-  const int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= c.R) return;
-  double2 sum = {0.0, 0.0};
-  for (int b = 0; b < nblk; ++b) {
-    const double2 p = partial[(int64_t)b * c.R + col];
-    sum.x += p.x;
-    sum.y += p.y;
-  }
+__global__ void __launch_bounds__(kRedThreads) k_norm_final(const double2* __restrict__ partial, int nblk, int rc, Cyc c) {
+  const double2 sum = block_sums(partial, nblk, c.R, rc);
+  const int64_t col = (int64_t)blockIdx.x * rc + threadIdx.x;
+  if (threadIdx.x >= rc || col >= c.R) return;
   const double nrm = sqrt(fmax(sum.x, 0.0));
   c.hn[col] = nrm;
   c.inv[col] = nrm > 0 ? 1.0 / nrm : 1.0;
@@ -580,19 +614,33 @@ __global__ void k_givens(Cyc c, int j, CondNext nx) {
   int active = 0;
   for (int64_t col = threadIdx.x; col < c.R; col += blockDim.x) {
     if (c.kuse[col] != 0) continue;
-    double2* h = c.H + ((size_t)col * m + j) * (m + 1);
-    for (int i = 0; i <= j; ++i) h[i] = c.hacc[(size_t)i * c.R + col];
-    h[j + 1] = {c.hn[col], 0.0};
+    // the running entry stays in registers, so the loads of a batch of rotations do not wait
+    // for the stores before them (through memory: 26 us a step of 64 columns)
+    double2* __restrict__ h = c.H + ((size_t)col * m + j) * (m + 1);
+    const double2* __restrict__ hacc = c.hacc + col;
     double2* cs = c.cs + (size_t)col * m;
     double2* sn = c.sn + (size_t)col * m;
-    for (int i = 0; i < j; ++i) {
-      const double2 a = h[i], b = h[i + 1];
-      const double2 t0 = z_cmul(cs[i], a), t1 = z_cmul(sn[i], b);
-      const double2 u0 = z_mul(sn[i], a), u1 = z_mul(cs[i], b);
-      h[i] = {t0.x + t1.x, t0.y + t1.y};
-      h[i + 1] = {u1.x - u0.x, u1.y - u0.y};
+    double2 a = hacc[0];
+    constexpr int kBatch = 8;
+    for (int i0 = 0; i0 < j; i0 += kBatch) {
+      double2 ci[kBatch], si[kBatch], bi[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (i0 + u < j) {
+          ci[u] = cs[i0 + u];
+          si[u] = sn[i0 + u];
+          bi[u] = hacc[(size_t)(i0 + u + 1) * c.R];
+        }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (i0 + u < j) {
+          const double2 t0 = z_cmul(ci[u], a), t1 = z_cmul(si[u], bi[u]);
+          const double2 u0 = z_mul(si[u], a), u1 = z_mul(ci[u], bi[u]);
+          h[i0 + u] = {t0.x + t1.x, t0.y + t1.y};
+          a = {u1.x - u0.x, u1.y - u0.y};
+        }
     }
-    const double2 a = h[j], b = h[j + 1];
+    const double2 b = {c.hn[col], 0.0};
     const double den = sqrt((a.x * a.x + a.y * a.y) + (b.x * b.x + b.y * b.y));
     const double2 cj = den > 0 ? double2{a.x / den, a.y / den} : double2{1.0, 0.0};
     const double2 sj = den > 0 ? double2{b.x / den, b.y / den} : double2{0.0, 0.0};
@@ -655,18 +703,18 @@ template <class VT>
 static void cgs2_graph(hb_factor_t f, const Dev& d, const Cyc& cyc, const VT* V, int nvec, VT* w, cudaStream_t s) {
   const int64_t nR = d.n * d.R;
   const bool fused = sub_dots_ok<VT>(nvec, d.R);   // the first update forms the second pass's dot products
-  const unsigned gfin = (unsigned)(((int64_t)nvec * d.R + 255) / 256);
+  const int nblk = red_blocks<VT>(d.n, d.R), rc = fin_cols(d.R);
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 0 || !fused)
-      k_dots_partial<VT><<<dim3(kRedBlocks, nvec), kRedThreads, 0, s>>>(V, nR, nvec, w, d.n, d.R, d.red_partial);
-    k_cgs_final<VT><<<gfin, 256, 0, s>>>(d.red_partial, kRedBlocks, nvec, cyc, pass);
+      k_dots_partial<VT><<<dim3(nblk, nvec), kRedThreads, 0, s>>>(V, nR, nvec, w, d.n, d.R, d.red_partial);
+    k_cgs_final<VT><<<fin_grid(d.R, nvec), kRedThreads, 0, s>>>(d.red_partial, nblk, rc, cyc, pass);
     if (pass == 0 && fused)
       launch_sub_dots<VT>(V, nR, nvec, (const VT*)cyc.cvec, w, d.n, d.R, d.red_partial, s);
     else
       k_sub_combo<VT><<<gsz(nR), 256, 0, s>>>(V, nR, nvec, (const VT*)cyc.cvec, w, d.n, d.R);
   }
-  k_dots_partial<VT><<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(w, 0, 1, w, d.n, d.R, d.red_partial);
-  k_norm_final<<<(unsigned)((d.R + 255) / 256), 256, 0, s>>>(d.red_partial, kRedBlocks, cyc);
+  k_dots_partial<VT><<<dim3(nblk, 1), kRedThreads, 0, s>>>(w, 0, 1, w, d.n, d.R, d.red_partial);
+  k_norm_final<<<fin_grid(d.R, 1), kRedThreads, 0, s>>>(d.red_partial, nblk, rc, cyc);
   k_scale_cols<VT, VT><<<gsz(nR), 256, 0, s>>>(w, cyc.inv, w, d.n, d.R);
   count_launch(f, fused ? 8 : 9);
 }
@@ -822,8 +870,8 @@ extern "C" int hb_gmres(hb_factor_t f, int op, const void* b_phys, void* x, int6
     f->prof.tag = -1;
     // start vector v_0 = r / ||r|| (split form: r <- L'^{-1} r first), g = beta e_1
     if (!mixed && (e = sweep_internal(f, PREC_F64, lo, r, R, s))) return e;
-    k_dots_partial<double2><<<dim3(kRedBlocks, 1), kRedThreads, 0, s>>>(r, 0, 1, r, n, R, d.red_partial);
-    k_cyc_start<<<gcol, 256, 0, s>>>(d.red_partial, kRedBlocks, cyc);
+    k_dots_partial<double2><<<dim3(red_blocks<double2>(n, R), 1), kRedThreads, 0, s>>>(r, 0, 1, r, n, R, d.red_partial);
+    k_cyc_start<<<fin_grid(R, 1), kRedThreads, 0, s>>>(d.red_partial, red_blocks<double2>(n, R), fin_cols(R), cyc);
     if (mixed) k_scale_cols<double2, float2><<<gsz(nR), 256, 0, s>>>(r, cyc.inv, V32, n, R);
     else k_scale_cols<double2, double2><<<gsz(nR), 256, 0, s>>>(r, cyc.inv, V, n, R);
     count_launch(f, 3);
