@@ -751,7 +751,7 @@ struct WideGrid {
     const int64_t need = (R + NC - 1) / NC;
     cw = (int)std::min<int64_t>(need, 128);
     cb = (unsigned)((need + cw - 1) / cw);
-    const int64_t fill = kWFill / (ops * cb * cw);
+    const int64_t fill = kWFill / (std::max<int64_t>(ops, 1) * cb * cw);
     ns = (int)std::max<int64_t>((64 + cw - 1) / cw, fill);
     ns = std::min(ns, std::min(kWSlots, kWThreads / cw));
   }

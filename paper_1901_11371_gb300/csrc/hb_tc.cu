@@ -20,8 +20,14 @@
 // copies it with one bulk copy, builds the A operand of each column tile from
 // the vectors (x / butterfly state) while converting and splitting, one
 // thread issues the MMAs (tcgen05.mma kind::f16, M = 128, N = 2 nn, K = 16
-// per instruction), and the four warps read the accumulator back
+// per instruction), and the warps read the accumulator back
 // (tcgen05.ld) and write the outputs (state entries / rows of y).
+// The loads of the A operand bound it: shared memory leaves one CTA on an SM
+// and no second A buffer, so the CTA has sixteen warps, four threads to a
+// column, to keep up to sixteen vector loads of each in flight, and the index
+// tables of a chunk are in shared memory first.  262,144 unknowns x 256
+// columns, entry + exit: 3.42 ms with one thread to a column and the tables
+// read from global memory, 1.60 ms now.
 // Every wait is bounded; a wait that gives up raises the factor's error flag.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -34,7 +40,8 @@ namespace hb {
 
 namespace {
 
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 512;
+constexpr int kTcShare = kTcThreads / 128;         // threads that share a column of the A operand
 constexpr int kTcMaxK = 128;                       // real-expanded inputs per chunk (2 x 64)
 constexpr int kTcMaxN = 128;                       // real-expanded outputs per chunk (2 x 64)
 constexpr int kTcABytes = 128 * kTcMaxK * 2;       // one bf16 A block (128 rows)
@@ -124,6 +131,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_jobs(TcArgs a) {
   uint64_t* mbar = (uint64_t*)(sm + kTcParts * kTcABytes + kTcParts * kTcBBytes);   // [0] B copy, [1] MMA done
   uint32_t* s_tmem = (uint32_t*)(mbar + 2);
   int* s_bad = (int*)(s_tmem + 1);
+  uint32_t* s_in = (uint32_t*)(s_bad + 1);                   // the chunk's input and output tables
+  uint32_t* s_out = s_in + kTcMaxK / 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const TcJob job = a.jobs[blockIdx.x];
   if (warp == 0) {
@@ -162,17 +171,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_jobs(TcArgs a) {
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                      ::"r"(su32(sB)), "l"(a.bpool + ch.boff), "r"(bbytes), "r"(su32(&mbar[0])) : "memory");
       }
+      for (int e = tid; e < ch.nk + ch.nn; e += kTcThreads) {
+        if (e < ch.nk) s_in[e] = a.tab[ch.in0 + e];
+        else s_out[e - ch.nk] = a.tab[ch.out0 + e - ch.nk];
+      }
+      __syncthreads();
       bool b_ready = false;
       for (int t = 0; t < ng; ++t) {
-        // ---- A operand of column tile g0 + t: thread = column m, 8 inputs per 16-byte store
-        const int64_t col = (int64_t)(g0 + t) * 128 + tid;
+        // ---- A operand of column tile g0 + t: thread = (column m, share), 8 inputs per 16-byte store
+        const int m = tid & 127, share = tid >> 7;
+        const int64_t col = (int64_t)(g0 + t) * 128 + m;
         const bool live = col < R;
-        const int rb = (tid >> 3) * (Kr >> 3) * 128 + (tid & 7) * 16;   // byte offset of row m, K group 0
-        for (int k0 = 0; k0 < ch.nk; k0 += 8) {
+        const int rb = (m >> 3) * (Kr >> 3) * 128 + (m & 7) * 16;   // byte offset of row m, K group 0
+#pragma unroll 2
+        for (int k0 = 8 * share; k0 < ch.nk; k0 += 8 * kTcShare) {
           float re[8], im[8];
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            const uint32_t e = a.tab[ch.in0 + k0 + u];
+            const uint32_t e = s_in[k0 + u];
             float2 v = make_float2(0.f, 0.f);
             if (live && e != kTcNone) v = (e & kTcVec) ? a.x[(int64_t)(e & ~kTcVec) * R + col] : a.st[(int64_t)e * R + col];
             re[u] = v.x;
@@ -227,20 +243,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_jobs(TcArgs a) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         // ---- epilogue of the tile's region after the chunk that completes it
         if (ch.flags & TC_LAST) {
-          const uint32_t rowaddr = tbase + ((uint32_t)(32 * warp) << 16) + (uint32_t)t * tile_cols + (uint32_t)ch.tcol;
+          // a warp reads the 32 lanes of its quarter; the four warps of a quarter share the outputs
+          const int quarter = warp & 3;
+          const uint32_t rowaddr = tbase + ((uint32_t)(32 * quarter) << 16) + (uint32_t)t * tile_cols + (uint32_t)ch.tcol;
           const uint32_t corr = 128u * (uint32_t)job.nreg;
-          for (int n0 = 0; n0 < ch.nn; n0 += 8) {
+          for (int n0 = 8 * (warp >> 2); n0 < ch.nn; n0 += 8 * kTcShare) {
             uint32_t vr[8], vi[8], cr[8], ci[8];
             tmem_ld8(rowaddr + (uint32_t)n0, vr);
             tmem_ld8(rowaddr + (uint32_t)(ch.nn + n0), vi);
             tmem_ld8(rowaddr + corr + (uint32_t)n0, cr);
             tmem_ld8(rowaddr + corr + (uint32_t)(ch.nn + n0), ci);
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-            const int64_t c = (int64_t)(g0 + t) * 128 + 32 * warp + lane;
+            const int64_t c = (int64_t)(g0 + t) * 128 + 32 * quarter + lane;
             if (c < R) {
 #pragma unroll
               for (int u = 0; u < 8; ++u) {
-                const uint32_t e = a.tab[ch.out0 + n0 + u];
+                const uint32_t e = s_out[n0 + u];
                 if (e == kTcNone) continue;
                 float2* d = (e & kTcVec) ? a.y + (int64_t)(e & ~kTcVec) * R + c : a.st + (int64_t)e * R + c;
                 *d = make_float2(__uint_as_float(vr[u]) + __uint_as_float(cr[u]),
