@@ -304,7 +304,223 @@ __global__ void __launch_bounds__(256) k_apply_exit(const DOuter* __restrict__ o
 }
 
 // ---------------------------------------------------------------------------
-// Column-parallel apply (R >= 2).  A CTA takes one op and up to cw * NC right-hand sides;
+// Two to kFewMax right-hand sides in FP32: a warp to an op, lanes over its outputs, RC columns
+// in a lane's registers.  With so few columns a staged chunk (below) is mostly barriers and idle
+// threads: 16,384 unknowns, complex64, 2 / 4 / 6 columns forward 117 / 119 / 137 us here against
+// 180 / 156 / 153 us, adjoint 104 / 106 / 130 against 201 / 166 / 160; at 8 columns the two meet
+// (150 / 142 against 148 / 149), at 12 the chunks lead (212 against 144).  In FP64 they lead
+// from 2 columns on (426 against 337 us), since here every lane repeats the column loop.
+// R = row stride of the [entry][R] layout, r0 = first RHS of this pass, rc = number of valid RHS
+// in the pass (<= RC).
+// ---------------------------------------------------------------------------
+constexpr int kFewMax = 8;
+
+// B side (k outputs) = gather + T * rest of the candidate vector cand =
+// concat(a0[0..ka0), a1[..]).  UTYPE_ADJ: the block is a row ID used in
+// adjoint (entries conj(T_ij) read from the U-type layout M[i*(c-k)+j]);
+// otherwise a column ID (V-type layout M[j*k+i]).
+template <class T, class F, int RC, bool UTYPE_ADJ>
+__device__ __forceinline__ void op_vlike(const F* __restrict__ M, const int16_t* __restrict__ idx, int k, int c,
+                                         const typename C2<T>::t* a0, int ka0, const typename C2<T>::t* a1,
+                                         typename C2<T>::t* out, int64_t R, int64_t r0, int rc, int lane) {
+  using C = typename C2<T>::t;
+  const int nr = c - k;
+  for (int i = lane; i < k; i += 32) {
+    C acc[RC];
+    const int qi = idx[i];
+    const C* src = (qi < ka0) ? a0 + (int64_t)qi * R : a1 + (int64_t)(qi - ka0) * R;
+#pragma unroll
+    for (int rr = 0; rr < RC; ++rr) acc[rr] = (rr < rc) ? src[r0 + rr] : mk<T>(0, 0);
+#pragma unroll 4
+    for (int j = 0; j < nr; ++j) {
+      C mij = UTYPE_ADJ ? ldf_conj<T>(M + (int64_t)i * nr + j) : ldf<T>(M + (int64_t)j * k + i);
+      const int pj = idx[k + j];
+      const C* s = (pj < ka0) ? a0 + (int64_t)pj * R : a1 + (int64_t)(pj - ka0) * R;
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr)
+        if (rr < rc) cfma(acc[rr], mij, s[r0 + rr]);
+    }
+#pragma unroll
+    for (int rr = 0; rr < RC; ++rr)
+      if (rr < rc) out[(int64_t)i * R + r0 + rr] = acc[rr];
+  }
+}
+
+// Contribution of one block to candidate entry r: VTYPE_ADJ: the block is a
+// column ID used in adjoint (conj(T_ij) from M[j*k+i]); otherwise a row ID
+// (U-type layout M[i*(c-k)+j]).
+template <class T, class F, int RC, bool VTYPE_ADJ>
+__device__ __forceinline__ void row_contrib(typename C2<T>::t (&acc)[RC], const F* __restrict__ M,
+                                            const int16_t* __restrict__ idx, int k, int c,
+                                            const typename C2<T>::t* y, int64_t R, int64_t r0, int rc, int r) {
+  using C = typename C2<T>::t;
+  const int code = idx[c + r];
+  if (code >= 0) {
+    const C* s = y + (int64_t)code * R + r0;
+#pragma unroll
+    for (int rr = 0; rr < RC; ++rr)
+      if (rr < rc) cadd(acc[rr], s[rr]);
+  } else {
+    const int j = -1 - code;
+    const int nr = c - k;
+#pragma unroll 4
+    for (int i = 0; i < k; ++i) {
+      C mij = VTYPE_ADJ ? ldf_conj<T>(M + (int64_t)j * k + i) : ldf<T>(M + (int64_t)i * nr + j);
+      const C* s = y + (int64_t)i * R + r0;
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr)
+        if (rr < rc) cfma(acc[rr], mij, s[rr]);
+    }
+  }
+}
+
+template <class T, class F, int RC>
+__device__ __forceinline__ void op_middle(const F* __restrict__ S, int kr, int kc, bool adj,
+                                          const typename C2<T>::t* in, typename C2<T>::t* out, int64_t R,
+                                          int64_t r0, int rc, int lane) {
+  using C = typename C2<T>::t;
+  const int nout = adj ? kc : kr, nin = adj ? kr : kc;
+  for (int o = lane; o < nout; o += 32) {
+    C acc[RC];
+#pragma unroll
+    for (int rr = 0; rr < RC; ++rr) acc[rr] = mk<T>(0, 0);
+#pragma unroll 4
+    for (int i = 0; i < nin; ++i) {
+      C s = adj ? ldf_conj<T>(S + (int64_t)o * kr + i) : ldf<T>(S + (int64_t)i * kr + o);
+      const C* v = in + (int64_t)i * R + r0;
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr)
+        if (rr < rc) cfma(acc[rr], s, v[rr]);
+    }
+#pragma unroll
+    for (int rr = 0; rr < RC; ++rr)
+      if (rr < rc) out[(int64_t)o * R + r0 + rr] = acc[rr];
+  }
+}
+
+// One inner item (two ID blocks or one middle block), one warp.
+template <class T, class F, int RC, bool ADJ>
+__device__ __forceinline__ void op_item(const DItem& it, const F* __restrict__ fp, const int16_t* __restrict__ ip,
+                                        typename C2<T>::t* st, int64_t R, int64_t r0, int rc, int lane) {
+  using C = typename C2<T>::t;
+  if (it.type == 1) {
+    const F* S = fp + it.blk[0].moff;
+    if (!ADJ) op_middle<T, F, RC>(S, it.b_k[0], it.a_k[0], false, st + (int64_t)it.a_off[0] * R, st + (int64_t)it.b_off[0] * R, R, r0, rc, lane);
+    else op_middle<T, F, RC>(S, it.b_k[0], it.a_k[0], true, st + (int64_t)it.b_off[0] * R, st + (int64_t)it.a_off[0] * R, R, r0, rc, lane);
+    return;
+  }
+  const bool to_b = (it.type == 0) != ADJ;   // V forward or U adjoint: A (candidates) -> B (skeletons)
+  if (to_b) {
+    const C* a0 = st + (int64_t)it.a_off[0] * R;
+    const C* a1 = st + (int64_t)it.a_off[1] * R;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const DBlk& b = it.blk[s];
+      if (it.type == 0)
+        op_vlike<T, F, RC, false>(fp + b.moff, ip + b.ioff, b.k, b.c, a0, it.a_k[0], a1, st + (int64_t)it.b_off[s] * R, R, r0, rc, lane);
+      else
+        op_vlike<T, F, RC, true>(fp + b.moff, ip + b.ioff, b.k, b.c, a0, it.a_k[0], a1, st + (int64_t)it.b_off[s] * R, R, r0, rc, lane);
+    }
+  } else {
+    const int c = it.a_k[0] + it.a_k[1];
+    for (int r = lane; r < c; r += 32) {
+      C acc[RC];
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr) acc[rr] = mk<T>(0, 0);
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const DBlk& b = it.blk[s];
+        if (it.type == 2)
+          row_contrib<T, F, RC, false>(acc, fp + b.moff, ip + b.ioff, b.k, b.c, st + (int64_t)it.b_off[s] * R, R, r0, rc, r);
+        else
+          row_contrib<T, F, RC, true>(acc, fp + b.moff, ip + b.ioff, b.k, b.c, st + (int64_t)it.b_off[s] * R, R, r0, rc, r);
+      }
+      C* dst = (r < it.a_k[0]) ? st + (int64_t)(it.a_off[0] + r) * R : st + (int64_t)(it.a_off[1] + r - it.a_k[0]) * R;
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr)
+        if (rr < rc) dst[r0 + rr] = acc[rr];
+    }
+  }
+}
+
+// Forward: block = column leaf j; warp w handles depths v = w, w+W, ...:
+// z_0 = V0 x_j.  Adjoint: block = row leaf i; y_0 = U0^H x_i.
+template <class T, class F, int RC, bool ADJ>
+__global__ void __launch_bounds__(256) k_few_enter(const DOuter* __restrict__ ops, int D, int64_t n0,
+                                                     const F* __restrict__ fp, const int16_t* __restrict__ ip,
+                                                     const typename C2<T>::t* __restrict__ x,
+                                                     typename C2<T>::t* st, int64_t R) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int64_t leaf = blockIdx.x;
+  const typename C2<T>::t* xl = x + leaf * n0 * R;
+  for (int v = warp; v < D; v += nw) {
+    const DOuter o = ops[leaf * D + v];
+    for (int64_t r0 = 0; r0 < R; r0 += RC) {
+      int rc = (int)(R - r0 < (int64_t)RC ? R - r0 : (int64_t)RC);
+      op_vlike<T, F, RC, ADJ>(fp + o.blk.moff, ip + o.blk.ioff, o.blk.k, o.blk.c, xl, (int)n0, xl,
+                              st + (int64_t)o.seg_off * R, R, r0, rc, lane);
+    }
+  }
+}
+
+template <class T, class F, int RC, bool ADJ>
+__global__ void __launch_bounds__(256) k_few_items(const DItem* __restrict__ items, const int32_t* __restrict__ idx,
+                                                     int count, const F* __restrict__ fp,
+                                                     const int16_t* __restrict__ ip, typename C2<T>::t* st,
+                                                     int64_t R) {
+  const int lane = threadIdx.x & 31;
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= count) return;
+  const DItem it = items[idx[w]];
+  for (int64_t r0 = 0; r0 < R; r0 += RC) {
+    int rc = (int)(R - r0 < (int64_t)RC ? R - r0 : (int64_t)RC);
+    op_item<T, F, RC, ADJ>(it, fp, ip, st, R, r0, rc, lane);
+  }
+}
+
+// Forward: block = row leaf i, thread = row r: y_r = sum_v (U0 y_0)_r + (A_leaf x_i)_r,
+// summed in the fixed order v = 0..D-1 then the dense leaf.  Adjoint: block =
+// column leaf j: (A^H x)_j = sum_v (V0^H z_0) + A_leaf^H x_j.
+template <class T, class F, int RC, bool ADJ>
+__global__ void __launch_bounds__(256) k_few_exit(const DOuter* __restrict__ ops, int D, int64_t n0,
+                                                    const F* __restrict__ fp, const int16_t* __restrict__ ip,
+                                                    const F* __restrict__ leafm,
+                                                    const typename C2<T>::t* __restrict__ x,
+                                                    const typename C2<T>::t* st, typename C2<T>::t* y,
+                                                    int64_t R) {
+  using C = typename C2<T>::t;
+  const int64_t leaf = blockIdx.x;
+  const F* A = leafm + leaf * n0 * n0;
+  const C* xl = x + leaf * n0 * R;
+  for (int r = threadIdx.x; r < n0; r += blockDim.x) {
+    for (int64_t r0 = 0; r0 < R; r0 += RC) {
+      int rc = (int)(R - r0 < (int64_t)RC ? R - r0 : (int64_t)RC);
+      C acc[RC];
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr) acc[rr] = mk<T>(0, 0);
+      for (int v = 0; v < D; ++v) {
+        const DOuter o = ops[leaf * D + v];
+        row_contrib<T, F, RC, ADJ>(acc, fp + o.blk.moff, ip + o.blk.ioff, o.blk.k, o.blk.c,
+                                   st + (int64_t)o.seg_off * R, R, r0, rc, r);
+      }
+#pragma unroll 4
+      for (int cc = 0; cc < n0; ++cc) {
+        C a = ADJ ? ldf_conj<T>(A + (int64_t)r * n0 + cc) : ldf<T>(A + (int64_t)cc * n0 + r);
+        const C* s = xl + (int64_t)cc * R + r0;
+#pragma unroll
+        for (int rr = 0; rr < RC; ++rr)
+          if (rr < rc) cfma(acc[rr], a, s[rr]);
+      }
+      C* dst = y + (leaf * n0 + r) * R + r0;
+#pragma unroll
+      for (int rr = 0; rr < RC; ++rr)
+        if (rr < rc) dst[rr] = acc[rr];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Column-parallel apply (R >= 2; FP32: more than kFewMax).  A CTA takes one op and up to cw * NC right-hand sides;
 // thread = (slot, column), and a slot owns chunks of KC outputs, which its threads keep in
 // registers for NC columns each while they walk the op's inputs once.  Vector rows are read
 // along the columns of the [entry][R] layout; a slot's coefficients [input][KC] and input
@@ -742,6 +958,33 @@ static int apply_one(const DevFactor& df, bool adj, const void* xv, void* yv, vo
   return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
 }
 
+template <class T, class F, int RC>
+static int apply_few(const DevFactor& df, bool adj, const void* xv, void* yv, int64_t R, void* stv,
+                      cudaStream_t s) {
+  using C = typename C2<T>::t;
+  const F* fp = (const F*)df.fpool;
+  const C* x = (const C*)xv;
+  C* y = (C*)yv;
+  C* st = (C*)stv;
+  int wpb = df.D < 8 ? df.D : 8;
+  if (!adj) k_few_enter<T, F, RC, false><<<(unsigned)df.m, 32 * wpb, 0, s>>>(df.vout, df.D, df.n0, fp, df.ipool, x, st, R);
+  else k_few_enter<T, F, RC, true><<<(unsigned)df.m, 32 * wpb, 0, s>>>(df.uout, df.D, df.n0, fp, df.ipool, x, st, R);
+  const std::vector<int32_t>& ptr = adj ? df.astep_ptr : df.step_ptr;
+  const int32_t* idx = adj ? df.astep_idx : df.step_idx;
+  for (int stp = 0; stp + 1 < (int)ptr.size(); ++stp) {
+    int cnt = ptr[stp + 1] - ptr[stp];
+    if (cnt <= 0) continue;
+    int blocks = (cnt + 7) / 8;
+    if (!adj) k_few_items<T, F, RC, false><<<blocks, 256, 0, s>>>(df.items, idx + ptr[stp], cnt, fp, df.ipool, st, R);
+    else k_few_items<T, F, RC, true><<<blocks, 256, 0, s>>>(df.items, idx + ptr[stp], cnt, fp, df.ipool, st, R);
+  }
+  int thr = (int)((df.n0 + 31) / 32 * 32);
+  if (thr > 256) thr = 256;
+  if (!adj) k_few_exit<T, F, RC, false><<<(unsigned)df.m, thr, 0, s>>>(df.uout, df.D, df.n0, fp, df.ipool, (const F*)df.leaf, x, st, y, R);
+  else k_few_exit<T, F, RC, true><<<(unsigned)df.m, thr, 0, s>>>(df.vout, df.D, df.n0, fp, df.ipool, (const F*)df.leaf, x, st, y, R);
+  return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
+}
+
 // Column threads cw and slots ns of the CTAs of `ops` ops: two warps at least, and with few ops
 // more slots, so that the step still fills the chip.
 struct WideGrid {
@@ -802,6 +1045,10 @@ static int apply_wide(const DevFactor& df, bool adj, const void* x, void* y, int
 template <class T, class F>
 static int apply_dispatch(const DevFactor& df, bool adj, const void* x, void* y, int64_t R, void* st,
                           cudaStream_t s) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (R > 1 && R <= 4) return apply_few<T, F, 4>(df, adj, x, y, R, st, s);
+    if (R > 1 && R <= kFewMax) return apply_few<T, F, 8>(df, adj, x, y, R, st, s);
+  }
   if (R > 1) return apply_wide<T, F>(df, adj, x, y, R, st, s);
   return apply_one<T, F>(df, adj, x, y, st, s);   // (the persistent kernel is tried first, in launch_apply)
 }

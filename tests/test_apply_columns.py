@@ -46,8 +46,8 @@ def test_apply(hb, name, form, bound):
     x = W.complex_gaussian(n, 9, 257).T.copy()
     b = W.complex_gaussian(n, 10, 257).T.copy()
     for op in (hb.HB_OP_N, hb.HB_OP_H):
-        ref = {c: hb.hb_host_apply(fh, x[c], op) for c in (0, 1, 2, 16, 31, 62, 63, 64, 129, 255, 256)}
-        for R in (1, 2, 3, 17, 32, 63, 64, 65, 130, 257):
+        ref = {c: hb.hb_host_apply(fh, x[c], op) for c in (0, 1, 2, 7, 8, 16, 31, 62, 63, 64, 129, 255, 256)}
+        for R in (1, 2, 3, 8, 9, 17, 32, 63, 64, 65, 130, 257):
             y = hb.hb_apply(f, torch.from_numpy(x[0] if R == 1 else x[:R]).cuda().to(dt), op)
             r = hb.hb_residual(f, torch.from_numpy(b[0] if R == 1 else b[:R]).cuda(),
                                torch.from_numpy(x[0] if R == 1 else x[:R]).cuda(), op)
