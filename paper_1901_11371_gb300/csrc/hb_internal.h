@@ -556,6 +556,11 @@ static_assert(sizeof(SwPhase) == 8, "phase entry");
 static_assert(sizeof(SwDesc) == 40, "batch descriptor");
 constexpr int kSwTileIn = 32 * 4, kSwTileCoef = kSwTileIn + 32 * 2;
 HB_HD inline int sw_pos(int e, int lane) { return (e >> 1) * 64 + lane * 2 + (e & 1); }
+// The kernel takes a resident tile's first kSwTilePairs entry pairs in registers, whether the
+// lanes (np pairs each) have them or not: pair i comes from this pair of the lane's inputs
+// (an absent one, of coefficient 0, from the first).
+constexpr int kSwTilePairs = 4;
+HB_HD inline int sw_tile_pair(int i, int np) { return i < np ? i : 0; }
 constexpr int kSwTriTab = 256;
 struct SwTriWarp {
   int n1, n0;

@@ -255,11 +255,10 @@ __device__ __forceinline__ void slot_async(const SwArgs& a, int32_t s, unsigned 
 // are held in registers, so that they can be fetched before the inputs exist; a longer
 // tile (a multiple of four entries) reads the rest as it goes.  Fewer than four pairs
 // (a phase of very few inputs): the absent ones have coefficient 0 and the lane's first inputs.
-constexpr int kTilePairs = 4;
 constexpr int kPairBytes = 32 * 16;   // one entry pair of all lanes
 template <int NC>
 struct Tile {
-  f2x2 cf[kTilePairs];
+  f2x2 cf[kSwTilePairs];
   unsigned va;              // shared address of the lane's first input
   unsigned coef;            // the lane's entries (shared memory)
   int np;                   // entry pairs per lane
@@ -271,21 +270,20 @@ struct Tile {
 template <int NC>
 __device__ __forceinline__ void tile_mac(const Tile<NC>& t, float2 (&s)[NC]) {
   Acc acc[NC];
-  f2x2 v[kTilePairs][NC];
-  const unsigned st = t.np >= kTilePairs ? 16 * NC : 0;
+  f2x2 v[kSwTilePairs][NC];
 #pragma unroll
-  for (int i = 0; i < kTilePairs; ++i)
+  for (int i = 0; i < kSwTilePairs; ++i)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) v[i][c] = lds_2(t.va + (i == 1 && t.np > 1 ? 16 * NC : i * st) + 16 * c);
+    for (int c = 0; c < NC; ++c) v[i][c] = lds_2(t.va + sw_tile_pair(i, t.np) * (16 * NC) + 16 * c);
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c].set(t.cf[0], v[0][c]);
 #pragma unroll
-  for (int i = 1; i < kTilePairs; ++i)
+  for (int i = 1; i < kSwTilePairs; ++i)
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[c].add(t.cf[i], v[i][c]);
-  if (t.np > kTilePairs) {
-    unsigned cp = t.coef + kTilePairs * kPairBytes, vp = t.va + kTilePairs * (16 * NC);
-    int i = kTilePairs;
+  if (t.np > kSwTilePairs) {
+    unsigned cp = t.coef + kSwTilePairs * kPairBytes, vp = t.va + kSwTilePairs * (16 * NC);
+    int i = kSwTilePairs;
 #pragma unroll 1
     for (; i + 1 < t.np; i += 2, cp += 2 * kPairBytes, vp += 2 * (16 * NC)) {
       f2x2 m[2], w[2][NC];
@@ -350,17 +348,15 @@ __device__ __forceinline__ void tile_open(Tile<NC>& t, unsigned gimg, int2 w, un
   t.dst = wr ? slot_addr<NC>(win, o & ~kSwAcc) + (NC == 2 && t.glog > 0 ? 16 * (lane & 1) : 0) : 0;
   t.coef = b + kSwTileCoef + 16 * lane;
   t.va = win + in * (8 * NC);
-  if (t.np >= kTilePairs) {
+  if (t.np >= kSwTilePairs) {
 #pragma unroll
-    for (int i = 0; i < kTilePairs; ++i) t.cf[i] = lds_2(t.coef + i * kPairBytes);
+    for (int i = 0; i < kSwTilePairs; ++i) t.cf[i] = lds_2(t.coef + i * kPairBytes);
   } else {
 #pragma unroll
-    for (int i = 0; i < kTilePairs; ++i) {
+    for (int i = 0; i < kSwTilePairs; ++i) {
       t.cf[i] = f2x2{0, 0};
-      lds_2_if(t.coef + i * kPairBytes, i < t.np && i < 2, t.cf[i]);
+      lds_2_if(t.coef + i * kPairBytes, i < t.np, t.cf[i]);
     }
-    // (three pairs: the third by itself)
-    if (t.np == 3) t.cf[2] = lds_2(t.coef + 2 * kPairBytes);
   }
 }
 // A resident phase's tiles b, b + stride, ... (< nb) of one warp, the first already in `t`.

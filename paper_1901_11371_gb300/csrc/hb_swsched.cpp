@@ -925,8 +925,10 @@ void host_sweep_sched(const PackedHost& ph, const SwSched& S, cplx* vec) {
               for (int e = 0; e < elen; e += 2) {
                 cplx v[2];
                 pair(cf + (t0 + sw_pos(e, l)) * S.coef_bytes, v);
+                // (a resident tile's inputs by the kernel's rule)
+                const int e2 = res && e < 2 * kSwTilePairs ? 2 * sw_tile_pair(e / 2, elen / 2) : e;
                 for (int q = 0; q < 2; ++q) {
-                  const int32_t at = in[32 * t + l] + e + q;
+                  const int32_t at = in[32 * t + l] + e2 + q;
                   acc += v[q] * (res ? win[at] : gv[at]);
                 }
               }

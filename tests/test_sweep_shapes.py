@@ -1,0 +1,96 @@
+"""Column-partitioned sweeps of coarse factors, whose phases are so small that their tiles take
+other shapes than those of fine ones.
+
+Bounds: a schedule with complex-FP32 coefficients, executed by the kernel's input rule, and the
+device's sweeps reproduce the packed program's own sweep to 1e-5 relative (the storage rounding
+and sums of a few hundred FP32 terms, as for the other sweep tests).
+"""
+import functools
+import math
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import workloads as W
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1901_11371_gb300", "csrc")
+# factors whose lowest butterflies have rank 5 or 6: tiles of three entry pairs
+RANK6 = [("arc", 1152, 72, 1e-3), ("arc", 1200, 75, 1e-2), ("strip", 1024, 128, 1e-2), ("arc", 1536, 96, 1e-2),
+         ("arc", 2048, 64, 1e-1)]
+
+
+@pytest.fixture(scope="session")
+def sweepcheck(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("g++ not available")
+    exe = str(tmp_path_factory.mktemp("sweepcheck") / "sweepcheck")
+    r = subprocess.run([gxx, "-O2", "-std=c++17", "-fopenmp", "-I", CSRC, os.path.join(ROOT, "tests", "sweepcheck.cpp"),
+                        os.path.join(CSRC, "hb_host.cpp"), os.path.join(CSRC, "hb_swsched.cpp"), "-o", exe],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+    def run(*args):
+        r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0, r.stdout[-2000:]
+        return r.stdout.split()
+    return run
+
+
+@functools.lru_cache(maxsize=None)
+def _hb():
+    from paper_1901_11371_gb300 import build
+    build.build()
+    import paper_1901_11371_gb300 as m
+    return m
+
+
+@pytest.fixture
+def hb_gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return _hb()
+
+
+def _geom(hb, curve, n):
+    if curve == "strip":
+        return hb.hb_geometry(hb.HB_STRIP, (0.0, 0.0, n / 20.0, 0.0), n)
+    return hb.hb_geometry(hb.HB_ARC, (n / 20.0 / math.pi, 0.0, math.pi), n)
+
+
+def _rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+def _check_sweeps(hb, curve, n, leaf, eps, options=0):
+    """All four sweeps on the device, with one column a CTA (1, 3) and with two (155)."""
+    import torch
+    g = _geom(hb, curve, n)
+    fh = hb.hb_factor_host(g, leaf, eps)
+    f = hb.hb_factor(g, leaf, eps, form=hb.HB_C64, options=options)
+    hb.hb_set_sweep_kernel(f, 1)
+    for R in (1, 3, 155):
+        b = W.complex_gaussian(n, 71 + R, R).T.copy()
+        bt = torch.from_numpy(b[0] if R == 1 else b).cuda().to(torch.complex64)
+        for w, (fn, op) in enumerate([(hb.hb_lower_solve, 0), (hb.hb_upper_solve, 0), (hb.hb_lower_solve, 1),
+                                      (hb.hb_upper_solve, 1)]):
+            x = fn(f, bt, op).cpu().numpy().astype(np.complex128).reshape(R, n)
+            for r in {0, R // 2, R - 1}:
+                assert _rel(x[r], hb.hb_host_sweep(fh, b[r], w)) <= 1e-5, (R, w, r)
+
+
+@pytest.mark.parametrize("curve,n,leaf,eps", RANK6)
+def test_tiles_of_three_pairs_by_the_kernels_rule(sweepcheck, curve, n, leaf, eps):
+    # (such tiles must be there, with a third pair that counts)
+    assert int(sweepcheck("tiles3", curve, n, leaf, eps)[1]) > 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("curve,n,leaf,eps", RANK6)
+def test_tiles_of_three_pairs_on_the_device(hb_gpu, curve, n, leaf, eps):
+    _check_sweeps(hb_gpu, curve, n, leaf, eps)
