@@ -567,6 +567,12 @@ struct SwTriWarp {
 };
 HB_HD inline int sw_tri_len(int r) { return r / 2 + 1; }   // column pairs of stored row r
 HB_HD inline bool sw_tri_live(int s, int j, bool hi) { return hi ? 2 * j <= s - 1 : 2 * j < s - 1; }   // row s-1-j / row j of pair j
+// Of a row's n steps, those that column group g takes of a triangle of even order s: its pair
+// g + 4 i of the last step may lie past the triangle's s / 2 pairs, where other rows stand, or none.
+HB_HD inline int sw_tri_take(int s, int g, int n) {
+  const int in = (s / 2 - g + 3) / 4;
+  return n < in ? n : in;
+}
 inline int sw_tri_warps(int s) { return ((s + 1) / 2 + 3) / 4; }
 inline SwTriWarp sw_tri_warp(int s, int v) {
   SwTriWarp w{0, 0};

@@ -510,7 +510,8 @@ __device__ __forceinline__ float2 tri_row(int n, unsigned coef, int r, unsigned 
   return acc.sum();
 }
 // The same for finite inputs of an even leaf size: nothing to mask (the coefficients beyond
-// the diagonal are zero), two steps in flight.  vp: the lane's first input, dv: bytes per step.
+// the diagonal are zero; n: the steps within the triangle), two steps in flight.  vp: the
+// lane's first input, dv: bytes per step.
 template <int NC>
 __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, int dv, int lane) {
   if (NC == 1) {
@@ -534,8 +535,8 @@ __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, 
 }
 template <int NC, bool EVEN, bool FAST>
 __device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsigned win, int n0, int warp, int lane) {
-  const int dv = (up ? -64 : 64) * NC;
-  const unsigned vp = slot_addr<NC>(win, a0 + (up ? s - 2 : 0)) + (NC == 2 ? 16 * (lane & 1) : 0) + ((lane >> 1) & 3) * (dv / 4);
+  const int dv = (up ? -64 : 64) * NC, g = (lane >> 1) & 3;
+  const unsigned vp = slot_addr<NC>(win, a0 + (up ? s - 2 : 0)) + (NC == 2 ? 16 * (lane & 1) : 0) + g * (dv / 4);
   const int nv = ((s + 1) / 2 + 3) / 4;
   float val[2] = {0.f, 0.f};
   unsigned dst[2] = {0, 0};   // 0: nothing to store
@@ -547,8 +548,9 @@ __device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsi
       const unsigned coef = T + kSwTriTab + (tw >> 16) * 256 + (lane >> 1) * 16;
       const int j = 4 * v + (lane >> 3);
       const int r1 = 2 * j <= s - 1 ? s - 1 - j : -1, r0 = 2 * j < s - 1 ? j : -1;
-      const float2 s1 = FAST ? tri_row_fast<NC>(n1, coef, vp, dv, lane) : tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
-      const float2 s0 = FAST ? tri_row_fast<NC>(nn0, coef + n1 * 256, vp, dv, lane)
+      const float2 s1 = FAST ? tri_row_fast<NC>(sw_tri_take(s, g, n1), coef, vp, dv, lane)
+                             : tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
+      const float2 s0 = FAST ? tri_row_fast<NC>(sw_tri_take(s, g, nn0), coef + n1 * 256, vp, dv, lane)
                              : tri_row<NC, EVEN>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
       // parting the sums over the lanes: a lane pair keeps one row, then one component
       constexpr int d1 = NC == 2 ? 2 : 1, d2 = 2 * d1;

@@ -6,6 +6,11 @@
 // CHECK = tiles3: prints how many resident tiles have three entry pairs whose third pair is
 // not zero (all four sweeps), and fails where a schedule with complex-FP32 coefficients,
 // executed with the kernel's input rule, is off the packed program's sweep by more than 1e-5.
+//
+//   sweepcheck triangle
+//
+// fails where a step of a triangle product of even order (2 .. 256, lower and upper) reads a
+// column that is not the triangle's.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -93,9 +98,32 @@ int tiles3(const PackedHost& ph) {
   return 0;
 }
 
+// the kernel's walk over a triangle without masks: warp v, its rows' steps, column groups
+int triangle() {
+  for (int s = 2; s <= 256; s += 2)
+    for (int v = 0; v < sw_tri_warps(s); ++v) {
+      const SwTriWarp tw = sw_tri_warp(s, v);
+      for (int n : {tw.n1, tw.n0})
+        for (int g = 0; g < 4; ++g)
+          for (int i = 0; i < sw_tri_take(s, g, n); ++i) {
+            const int p = g + 4 * i, lower = 2 * p, upper = s - 2 - 2 * p;
+            if (lower + 1 >= s || upper < 0) { std::printf("FAIL: order %d, pair %d\n", s, p); return 1; }
+          }
+      // and no pair of a row is left out
+      for (int j = 4 * v; j < 4 * v + 4; ++j)
+        for (bool hi : {true, false})
+          if (sw_tri_live(s, j, hi))
+            for (int p = 0; p < sw_tri_len(hi ? s - 1 - j : j); ++p)
+              if (p / 4 >= sw_tri_take(s, p % 4, hi ? tw.n1 : tw.n0)) { std::printf("FAIL: order %d without pair %d\n", s, p); return 1; }
+    }
+  std::printf("OK\n");
+  return 0;
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
+  if (argc == 2 && !std::strcmp(argv[1], "triangle")) return triangle();
   if (argc != 6) return 2;
   const std::string what = argv[1];
   const PackedHost ph = pack(argv[2], std::atoll(argv[3]), std::atoll(argv[4]), std::atof(argv[5]));

@@ -1,5 +1,6 @@
-"""Column-partitioned sweeps of coarse factors, whose phases are so small that their tiles take
-other shapes than those of fine ones.
+"""Column-partitioned sweeps of factors whose phases or triangles take other shapes than the usual:
+coarse ones, whose phases are so small that tiles have fewer entries, and sweep leaves whose
+order is no multiple of eight.
 
 Bounds: a schedule with complex-FP32 coefficients, executed by the kernel's input rule, and the
 device's sweeps reproduce the packed program's own sweep to 1e-5 relative (the storage rounding
@@ -94,3 +95,14 @@ def test_tiles_of_three_pairs_by_the_kernels_rule(sweepcheck, curve, n, leaf, ep
 @pytest.mark.parametrize("curve,n,leaf,eps", RANK6)
 def test_tiles_of_three_pairs_on_the_device(hb_gpu, curve, n, leaf, eps):
     _check_sweeps(hb_gpu, curve, n, leaf, eps)
+
+
+def test_triangles_read_their_own_columns(sweepcheck):
+    sweepcheck("triangle")
+
+
+# sweep leaves of 68, 100, 84, 108 and 100 rows
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,leaf", [(1088, 34), (1600, 50), (1344, 42), (1728, 54), (1600, 100)])
+def test_sweep_leaves_off_a_multiple_of_eight_on_the_device(hb_gpu, n, leaf):
+    _check_sweeps(hb_gpu, "arc", n, leaf, 1e-6)
