@@ -489,6 +489,11 @@ enum SwGroupFlag : int32_t {
   SWG_BEGIN = 8,    // group: load the window rows of vector rows [beg_lo, beg_hi) first
   SWG_ENDRUN = 16,  // group: write vector rows [end_lo, end_hi) back after its last phase
 };
+// SwGroupHdr::flags of a run's first group, upper bits: the window slots that the run uses (rows,
+// then state).  The run starts with all of them written, those without a row with zeros: tiles
+// also read slots that no stage writes (the pad of an odd input list, coefficient 0), and
+// global phases leave their gathered entries there, both columns of a CTA side by side.
+constexpr int kSwGroupSlots = 8;
 enum SwPhaseFlag : int32_t {
   SWP_END = 1,      // the phase ends with this part: barrier among the compute warps
   SWP_TRI = 2,      // one triangle batch, taken by all compute warps

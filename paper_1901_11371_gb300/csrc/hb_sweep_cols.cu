@@ -14,8 +14,9 @@
 //     that allocated ring space and looked at every release took about a thousand
 //     cycles per group, which bounded the kernel);
 //   * resident runs (subtrees whose rows and live butterfly state fit the 96 KB
-//     window) start by loading their rows into shared memory and end by
-//     writing them back; inside them every phase reads and writes the window;
+//     window) start by loading their rows into shared memory, and zeros into the
+//     rest of what they use, and end by writing the rows back; inside them every
+//     phase reads and writes the window;
 //   * global phases (stages of the large butterflies) read and write the
 //     vector rows and a CTA-private butterfly state in global memory; every batch
 //     belongs to one warp, which gathers its inputs (cp.async, the next batch's in
@@ -608,8 +609,6 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
     s_issued = 0;
     s_odd = -1;
   }
-  // (the unused slots that pad odd input lists are multiplied by zero: no NaN may stand there)
-  for (int e = threadIdx.x; e < kSwWinBytes / 16; e += blockDim.x) sts_f4(win_a + 16 * e, 0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   if (warp == kSwWarps) {
     // ---- producer: every group of the schedule into its place in the ring, one lane each,
@@ -751,6 +750,20 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
       // ---- a resident run: groups g .. g + aux - 1
       const int gend = g + aux, unit = g;
       const int2 rows = lds_i2(gimg + 8);   // the run's rows [lo, hi)
+      {
+        // its slots without a row: zero (they are read as inputs of coefficient 0)
+        const int nrow = rows.y - rows.x, leaves = (n0 & 1) ? nrow / n0 : 0, rslots = nrow + leaves;
+        const unsigned lo = win_a + rslots * (8 * NC), hi = win_a + (H.y >> kSwGroupSlots) * (8 * NC);
+        for (unsigned d = lo + 16 * t; d < hi; d += 16 * kSwWarps * 32) sts_f4(d, 0.f, 0.f, 0.f, 0.f);
+        for (int l = t; l < leaves; l += kSwWarps * 32) {
+          const unsigned d = slot_addr<NC>(win_a, l * (n0 + 1) + n0);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            sts_f(d + 16 * c, 0.f);
+            sts_f(d + 16 * c + 8, 0.f);
+          }
+        }
+      }
 #pragma unroll 4
       for (int r = t; r < rows.y - rows.x; r += kSwWarps * 32) {
         const float2* src = xb + (int64_t)(rows.x + r) * a.R;

@@ -806,6 +806,7 @@ void build_sweep_sched(const PackedHost& ph, int which, int coef_bytes, int win_
       std::memcpy(&H, hb, sizeof(H));
       if (!(H.flags & SWG_BEGIN)) { S.ok = false; S.why = "resident run without its first group"; return; }
       H.aux = (int32_t)(S.groups.size() - run_g0);
+      H.flags |= (int32_t)(row_slots + 2 * stage) << kSwGroupSlots;
       std::memcpy(hb, &H, sizeof(H));
       // phase by phase: the warps that compute it, the barrier after it
       int32_t* prev = nullptr;
@@ -869,8 +870,10 @@ void host_sweep_sched(const PackedHost& ph, const SwSched& S, cplx* vec) {
     const uint8_t* gb = S.image.data() + G.img;
     SwGroupHdr H;
     std::memcpy(&H, gb, sizeof(H));
-    if (H.flags & SWG_BEGIN)
+    if (H.flags & SWG_BEGIN) {
+      std::fill(win.begin(), win.begin() + (H.flags >> kSwGroupSlots), cplx(0.0, 0.0));
       for (int32_t r = H.beg_lo; r < H.beg_hi; ++r) win[sw_row_slot(r - H.beg_lo, n0)] = vec[r];
+    }
     const bool res = (H.flags & SWG_RES) != 0;
     for (int32_t k = 0; k < H.nph; ++k) {
       SwPhase PH;
@@ -957,7 +960,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
   const int cb = S.coef_bytes;
   int64_t run_left = 0;   // groups of the current resident run still to come
   int64_t glob_left = 0;  // groups of the current global phase still to come
-  int32_t win_rows = 0;   // window slots of the run's rows
+  int32_t win_rows = 0, run_slots = 0;   // window slots of the run's rows; all that it uses
   // per window slot: the last resident phase that wrote / read it (a resident
   // phase's batches run concurrently on the compute warps, so no slot may be
   // written twice in a phase, nor written and read by the same phase)
@@ -987,7 +990,8 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
         run_left = H.aux;
         if (H.beg_lo < 0 || H.beg_hi <= H.beg_lo || H.beg_hi > n || H.beg_lo % n0 || H.beg_hi % n0) return "run rows";
         win_rows = (H.beg_hi - H.beg_lo) / n0 * sw_leaf_stride(n0);
-        if (win_rows > S.win_slots) return "run rows";
+        run_slots = H.flags >> kSwGroupSlots;
+        if (win_rows > run_slots || run_slots > S.win_slots || (run_slots & 1)) return "run rows";
       } else if (H.flags & SWG_BEGIN) {
         return "BEGIN inside a run";
       }
@@ -1063,7 +1067,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
         for (int32_t r = 0; r < D.nrows; ++r) {
           if (!res && (out[r] & kSwAcc)) return "global row that adds in place";
           const int32_t o = out[r] & ~kSwAcc;
-          if (res ? (o < 0 || o >= S.win_slots) : (o < 0 || o >= n + ph.state_len)) return "output slot";
+          if (res ? (o < 0 || o >= run_slots) : (o < 0 || o >= n + ph.state_len)) return "output slot";
           if (res) {
             if (wstamp[o] == pid) return "window slot written twice in one phase";
             if (rstamp[o] == pid) return "window slot read and written in one phase";
@@ -1074,7 +1078,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
           const int elen = res ? D.elen : e0[t + 1] - e0[t];
           for (int l = 0; l < 32; ++l) {
             const int32_t i0 = in[32 * t + l];
-            if (i0 < 0 || i0 + elen > (res ? S.win_slots : D.a0 ? D.a0 : D.ngl)) return "input slot";
+            if (i0 < 0 || i0 + elen > (res ? run_slots : D.a0 ? D.a0 : D.ngl)) return "input slot";
             if (res)
               for (int32_t i = i0; i < i0 + elen; ++i) {
                 if (wstamp[i] == pid) return "window slot read and written in one phase";

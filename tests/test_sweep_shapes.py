@@ -1,6 +1,6 @@
 """Column-partitioned sweeps of factors whose phases or triangles take other shapes than the usual:
 coarse ones, whose phases are so small that tiles have fewer entries, and sweep leaves whose
-order is no multiple of eight.
+order is no multiple of eight; and what a NaN in one right-hand side reaches.
 
 Bounds: a schedule with complex-FP32 coefficients, executed by the kernel's input rule, and the
 device's sweeps reproduce the packed program's own sweep to 1e-5 relative (the storage rounding
@@ -106,3 +106,28 @@ def test_triangles_read_their_own_columns(sweepcheck):
 @pytest.mark.parametrize("n,leaf", [(1088, 34), (1600, 50), (1344, 42), (1728, 54), (1600, 100)])
 def test_sweep_leaves_off_a_multiple_of_eight_on_the_device(hb_gpu, n, leaf):
     _check_sweeps(hb_gpu, "arc", n, leaf, 1e-6)
+
+
+# (factors with global phases before resident runs)
+@pytest.mark.parametrize("check,n,leaf", [("nan", 16384, 64), ("nan_small", 1600, 25), ("nan_small", 1600, 50)])
+def test_nan_stays_in_its_column_by_the_kernels_rule(sweepcheck, check, n, leaf):
+    sweepcheck(check, "arc", n, leaf, 1e-6)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,leaf,row,small", [(16384, 64, 8192, False), (1600, 25, 5, True), (1600, 50, 5, True)])
+def test_nan_stays_in_its_column_on_the_device(hb_gpu, n, leaf, row, small):
+    # 160 columns, two a CTA.  The other columns see the same sums in the same order: equal.
+    import torch
+    hb = hb_gpu
+    f = hb.hb_factor(_geom(hb, "arc", n), leaf, 1e-6, form=hb.HB_C64, options=hb.HB_OPT_SWEEP_WINDOW_MIN if small else 0)
+    hb.hb_set_sweep_kernel(f, 1)
+    R, q = 160, 7
+    b = torch.from_numpy(W.complex_gaussian(n, 90, R).T.copy()).cuda().to(torch.complex64)
+    bad = b.clone()
+    bad[q, row] = complex(float("nan"), 0.0)
+    others = [r for r in range(R) if r != q]
+    for fn, op in [(hb.hb_lower_solve, 0), (hb.hb_upper_solve, 0), (hb.hb_lower_solve, 1), (hb.hb_upper_solve, 1)]:
+        clean, x = fn(f, b, op), fn(f, bad, op)
+        assert torch.equal(x[others], clean[others])
+        assert torch.isnan(torch.view_as_real(x[q, row])).any()
