@@ -186,6 +186,14 @@ __device__ __forceinline__ void sts_f(unsigned a, float v) {
 __device__ __forceinline__ void sts_f4(unsigned a, float x, float y, float z, float w) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
+// image data, staged (shared address) or where it stands in global memory
+__device__ __forceinline__ f2x2 img_2(unsigned a) { return lds_2(a); }
+__device__ __forceinline__ f2x2 img_2(const uint8_t* p) {
+  const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
+  return f2x2{v.x, v.y};
+}
+__device__ __forceinline__ int img_i(unsigned a) { return lds_i(a); }
+__device__ __forceinline__ int img_i(const uint8_t* p) { return __ldg(reinterpret_cast<const int*>(p)); }
 __device__ __forceinline__ f2x ffma2(f2x a, f2x b, f2x c) {   // two FP32 multiply-adds
   f2x d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
@@ -223,6 +231,16 @@ struct Acc {
     return make_float2((lo(rr) + hi(rr)) - (lo(ii) + hi(ii)), (lo(ri) + hi(ri)) + (lo(ir) + hi(ir)));
   }
 };
+
+// inputs v as the coefficients m take them: nothing where a coefficient is zero (0 times a
+// foreign Inf or NaN would be NaN)
+__device__ __forceinline__ f2x2 masked(const f2x2& m, f2x2 v) {
+  const f2x k = (lo(m.a) == 0.f && lo(m.b) == 0.f ? 0ull : 0xffffffffull) |
+                (hi(m.a) == 0.f && hi(m.b) == 0.f ? 0ull : 0xffffffffull << 32);
+  v.a &= k;
+  v.b &= k;
+  return v;
+}
 
 // address of a global slot: a vector row (this CTA's columns of x) or a
 // CTA-private state entry
@@ -466,9 +484,9 @@ __device__ __forceinline__ void run_batch(const SwArgs& a, unsigned desc, unsign
 // every lane has the same 17 steps at order 128, a step's coefficients are consecutive,
 // its inputs four neighbouring column pairs that all row pairs share, and a row's sum
 // needs two shuffle rounds and no other warp; one barrier separates the reads of the rows
-// from their replacement.  Where the run's rows were not all finite, inputs beyond a row's
-// diagonal are masked (0 times a foreign row's Inf would be NaN).  EVEN: the window's slots
-// pair up like the columns (even leaf size).
+// from their replacement.  FAST: without masks; else inputs beyond a row's diagonal are masked
+// (0 times a foreign row's Inf would be NaN).  EVEN: the window's slots pair up like the columns
+// (even leaf size).
 template <int NC, bool EVEN>
 __device__ __forceinline__ f2x2 tri_input(unsigned win, int a0, int s, bool up, int p, int c, int n0) {
   if constexpr (EVEN) {
@@ -491,8 +509,8 @@ __device__ __forceinline__ f2x2 tri_input(unsigned win, int a0, int s, bool up, 
   }
 }
 // row r's sum over steps [0, n) (r < 0: no such row); coef: the lane's first coefficient
-template <int NC, bool EVEN>
-__device__ __forceinline__ float2 tri_row(int n, unsigned coef, int r, unsigned win, int a0, int s, bool up, int n0, int lane) {
+template <int NC, bool EVEN, class P>
+__device__ __forceinline__ float2 tri_row(int n, P coef, int r, unsigned win, int a0, int s, bool up, int n0, int lane) {
   const int g = (lane >> 1) & 3, c = NC == 2 ? lane & 1 : 0;
   // with one column the lane takes every second step
   const int i0 = NC == 2 ? 0 : lane & 1, di = NC == 2 ? 1 : 2;
@@ -506,13 +524,13 @@ __device__ __forceinline__ float2 tri_row(int n, unsigned coef, int r, unsigned 
     const f2x mask = two ? ~0ull : up ? 0xffffffffull << 32 : 0xffffffffull;
     v.a &= mask;
     v.b &= mask;
-    acc.add(lds_2(coef + i * 256), v);
+    acc.add(img_2(coef + i * 256), v);
   }
   return acc.sum();
 }
-// The same for finite inputs of an even leaf size: nothing to mask (the coefficients beyond
-// the diagonal are zero; n: the steps within the triangle), two steps in flight.  vp: the
-// lane's first input, dv: bytes per step.
+// The same without masks, for an even leaf size (the coefficients beyond the diagonal are zero;
+// n: the steps within the triangle), two steps in flight.  vp: the lane's first input, dv: bytes
+// per step.
 template <int NC>
 __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, int dv, int lane) {
   if (NC == 1) {
@@ -534,8 +552,8 @@ __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, 
   if (i < n) acc.add(lds_2(cp), lds_2(vp));
   return acc.sum();
 }
-template <int NC, bool EVEN, bool FAST>
-__device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsigned win, int n0, int warp, int lane) {
+template <int NC, bool EVEN, bool FAST, class P>
+__device__ __forceinline__ void run_tri(int s, int a0, bool up, P T, unsigned win, int n0, int warp, int lane) {
   const int dv = (up ? -64 : 64) * NC, g = (lane >> 1) & 3;
   const unsigned vp = slot_addr<NC>(win, a0 + (up ? s - 2 : 0)) + (NC == 2 ? 16 * (lane & 1) : 0) + g * (dv / 4);
   const int nv = ((s + 1) / 2 + 3) / 4;
@@ -545,14 +563,18 @@ __device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsi
   for (int h = 0; h < 2; ++h) {
     const int v = warp + kSwWarps * h;
     if (v < nv) {
-      const int tw = lds_i(T + 4 * v), n1 = (tw >> 8) & 0xff, nn0 = tw & 0xff;
-      const unsigned coef = T + kSwTriTab + (tw >> 16) * 256 + (lane >> 1) * 16;
+      const int tw = img_i(T + 4 * v), n1 = (tw >> 8) & 0xff, nn0 = tw & 0xff;
+      const P coef = T + (kSwTriTab + (tw >> 16) * 256 + (lane >> 1) * 16);
       const int j = 4 * v + (lane >> 3);
       const int r1 = 2 * j <= s - 1 ? s - 1 - j : -1, r0 = 2 * j < s - 1 ? j : -1;
-      const float2 s1 = FAST ? tri_row_fast<NC>(sw_tri_take(s, g, n1), coef, vp, dv, lane)
-                             : tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
-      const float2 s0 = FAST ? tri_row_fast<NC>(sw_tri_take(s, g, nn0), coef + n1 * 256, vp, dv, lane)
-                             : tri_row<NC, EVEN>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
+      float2 s1, s0;
+      if constexpr (FAST) {
+        s1 = tri_row_fast<NC>(sw_tri_take(s, g, n1), coef, vp, dv, lane);
+        s0 = tri_row_fast<NC>(sw_tri_take(s, g, nn0), coef + n1 * 256, vp, dv, lane);
+      } else {
+        s1 = tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
+        s0 = tri_row<NC, EVEN>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
+      }
       // parting the sums over the lanes: a lane pair keeps one row, then one component
       constexpr int d1 = NC == 2 ? 2 : 1, d2 = 2 * d1;
       const bool b1 = lane & d1, b2 = lane & d2;
@@ -577,10 +599,91 @@ __device__ __forceinline__ void run_tri(int s, int a0, bool up, unsigned T, unsi
     if (dst[h]) sts_f(dst[h], val[h]);
 }
 
-// (out of line: rarely taken)
-template <int NC, bool EVEN>
-__device__ __noinline__ void run_tri_masked(int s, int a0, bool up, unsigned T, unsigned win, int n0, int warp, int lane) {
-  run_tri<NC, EVEN, false>(s, a0, up, T, win, n0, warp, lane);
+// Rows [lo, hi) of the CTA's columns (xb, row stride R) into the window, all compute warps, and
+// zeros into its slots without a row, up to `slots` (they are read as inputs of coefficient 0).
+template <int NC>
+__device__ __forceinline__ void load_rows(const float2* xb, int64_t R, int lo, int hi, int slots, int n0, int ncol,
+                                          unsigned win, int t) {
+  const int nrow = hi - lo, leaves = (n0 & 1) ? nrow / n0 : 0;
+  const unsigned z1 = win + slots * (8 * NC);
+  for (unsigned d = win + (nrow + leaves) * (8 * NC) + 16 * t; d < z1; d += 16 * kSwWarps * 32) sts_f4(d, 0.f, 0.f, 0.f, 0.f);
+  for (int l = t; l < leaves; l += kSwWarps * 32) {
+    const unsigned d = slot_addr<NC>(win, l * (n0 + 1) + n0);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      sts_f(d + 16 * c, 0.f);
+      sts_f(d + 16 * c + 8, 0.f);
+    }
+  }
+#pragma unroll 4
+  for (int r = t; r < nrow; r += kSwWarps * 32) {
+    const float2* src = xb + (int64_t)(lo + r) * R;
+    const unsigned d = slot_addr<NC>(win, sw_row_slot(r, n0));
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const float2 v = c < ncol ? __ldcg(src + c) : make_float2(0.f, 0.f);
+      sts_f(d + 16 * c, v.x);
+      sts_f(d + 16 * c + 8, v.y);
+    }
+  }
+}
+
+// A resident run once more from its rows, with every zero coefficient masked: for a run whose
+// rows came out non-finite, since a foreign Inf or NaN times zero (a neighbour's slot, a row
+// beyond the diagonal) may have made them so.  All compute warps; the groups are read where they
+// stand in global memory (the ring has moved on), the sums have the order of the run proper.
+template <int NC>
+__device__ __forceinline__ void redo_run(const uint8_t* image, const SwGroup* groups, int ngroup, const float2* xb, int64_t R,
+                                      int n0, int ncol, unsigned win, int warp, int lane) {
+  for (int g = 0; g < ngroup; ++g) {
+    const uint8_t* img = image + groups[g].img;
+    const SwGroupHdr H = *reinterpret_cast<const SwGroupHdr*>(img);
+    if (g == 0) {
+      load_rows<NC>(xb, R, H.beg_lo, H.beg_hi, H.flags >> kSwGroupSlots, n0, ncol, win, 32 * warp + lane);
+      all_sync();
+    }
+    const SwDesc* desc = reinterpret_cast<const SwDesc*>(img + H.off_desc);
+    for (int k = 0; k < H.nph; ++k) {
+      const SwPhase PH = reinterpret_cast<const SwPhase*>(img + 32)[k];
+      if (PH.flags & SWP_TRI) {
+        const uint8_t* T = img + desc->off;
+        const bool up = (PH.flags & SWP_UPPER) != 0;
+        if (n0 & 1) run_tri<NC, false, false>(desc->nrows, desc->a0, up, T, win, n0, warp, lane);
+        else run_tri<NC, true, false>(desc->nrows, desc->a0, up, T, win, n0, warp, lane);
+      } else {
+        for (int b = warp; b < PH.nb; b += kSwWarps) {
+          const SwDesc& D = desc[b];
+          const uint8_t* data = img + D.off;
+          const int glog = D.glog, in = reinterpret_cast<const int16_t*>(data + kSwTileIn)[lane];
+          unsigned vp = win + in * (8 * NC);
+          const uint8_t* cp = data + kSwTileCoef + 16 * lane;
+          Acc acc[NC];
+          for (int i = 0; i < D.elen / 2; ++i, cp += kPairBytes, vp += 16 * NC) {
+            const f2x2 m = img_2(cp);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c].add(m, masked(m, lds_2(vp + 16 * c)));
+          }
+          float2 s[NC];
+#pragma unroll
+          for (int c = 0; c < NC; ++c) s[c] = acc[c].sum();
+          tile_reduce<NC>(s, glog, lane);
+          if (tile_writer<NC>(D.trows, glog, lane)) {
+            const int o = reinterpret_cast<const int32_t*>(data)[lane >> glog];
+            const unsigned dst = slot_addr<NC>(win, o & ~kSwAcc) + (NC == 2 && glog > 0 ? 16 * (lane & 1) : 0);
+#pragma unroll
+            for (int c = 0; c < (NC == 2 && glog == 0 ? NC : 1); ++c) {
+              const unsigned d = dst + 16 * c;
+              const float2 old = o < 0 ? make_float2(lds_f(d), lds_f(d + 8)) : make_float2(0.f, 0.f);
+              sts_f(d, old.x + s[c].x);
+              sts_f(d + 8, old.y + s[c].y);
+            }
+          }
+        }
+      }
+      desc += PH.nb;
+      if (PH.flags & SWP_END) all_sync();
+    }
+  }
 }
 
 template <int NC>
@@ -592,7 +695,7 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
   __shared__ __align__(8) uint64_t s_mbar[kSwFlight];    // group in the slot has arrived
   __shared__ __align__(8) uint64_t s_free[kSwFlight];    // every compute warp is done with it
   __shared__ int s_abort, s_issued;
-  __shared__ int s_odd;    // the last run (its first group) that loaded a non-finite row
+  __shared__ int s_redo;   // the compute warps are busy with a run's second pass
   const unsigned ring_a = su32(smem), win_a = ring_a + kSwRingBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t lb = a.col0 + (int64_t)blockIdx.x * NC;
@@ -607,7 +710,7 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     s_abort = 0;
     s_issued = 0;
-    s_odd = -1;
+    s_redo = 0;
   }
   __syncthreads();
   if (warp == kSwWarps) {
@@ -643,7 +746,8 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
         const int adv = busy ? __ffs(busy) - 1 : 32;
         done += adv;
         if (adv == 0) {
-          if (__any_sync(0xffffffffu, ++spins > a.spin_limit || *(volatile int*)&s_abort)) {
+          if (!*(volatile int*)&s_redo) ++spins;   // (a second pass takes its time, but ends)
+          if (__any_sync(0xffffffffu, spins > a.spin_limit || *(volatile int*)&s_abort)) {
             if (lane == 0) {
               atomicExch(&s_abort, 1);
               s_issued = issued;
@@ -748,34 +852,9 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
         continue;
       }
       // ---- a resident run: groups g .. g + aux - 1
-      const int gend = g + aux, unit = g;
+      const int gend = g + aux, g_first = g;
       const int2 rows = lds_i2(gimg + 8);   // the run's rows [lo, hi)
-      {
-        // its slots without a row: zero (they are read as inputs of coefficient 0)
-        const int nrow = rows.y - rows.x, leaves = (n0 & 1) ? nrow / n0 : 0, rslots = nrow + leaves;
-        const unsigned lo = win_a + rslots * (8 * NC), hi = win_a + (H.y >> kSwGroupSlots) * (8 * NC);
-        for (unsigned d = lo + 16 * t; d < hi; d += 16 * kSwWarps * 32) sts_f4(d, 0.f, 0.f, 0.f, 0.f);
-        for (int l = t; l < leaves; l += kSwWarps * 32) {
-          const unsigned d = slot_addr<NC>(win_a, l * (n0 + 1) + n0);
-#pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            sts_f(d + 16 * c, 0.f);
-            sts_f(d + 16 * c + 8, 0.f);
-          }
-        }
-      }
-#pragma unroll 4
-      for (int r = t; r < rows.y - rows.x; r += kSwWarps * 32) {
-        const float2* src = xb + (int64_t)(rows.x + r) * a.R;
-        const unsigned d = slot_addr<NC>(win_a, sw_row_slot(r, n0));
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const float2 v = c < ncol ? __ldcg(src + c) : make_float2(0.f, 0.f);
-          if (!isfinite(v.x) || !isfinite(v.y)) *(volatile int*)&s_odd = unit;
-          sts_f(d + 16 * c, v.x);
-          sts_f(d + 16 * c + 8, v.y);
-        }
-      }
+      load_rows<NC>(xb, a.R, rows.x, rows.y, H.y >> kSwGroupSlots, n0, ncol, win_a, t);
       const int set = warp >= kSwSet ? SWP_SET1 : 0, wset = warp & (kSwSet - 1);
       bool hand = false, sync = true;   // the previous phase hands over to this one's set / all warps meet
       unsigned hid = 3;       // barrier of the next hand-over (3 and 4 in turn)
@@ -819,8 +898,7 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
             if (!bad) {
               const int toff = lds_i(desc), s = lds_i(desc + 8), a0 = lds_i(desc + 20);
               const bool up = (PH.y & SWP_UPPER) != 0;
-              if (n0 & 1) run_tri_masked<NC, false>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
-              else if (*(volatile int*)&s_odd == unit) run_tri_masked<NC, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+              if (n0 & 1) run_tri<NC, false, false>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
               else run_tri<NC, true, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
             } else {
               all_sync();   // the barrier inside the triangle product
@@ -853,6 +931,18 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
         }
       }
       all_sync();   // the run's last phase is done
+      // An Inf or NaN that met a zero coefficient has made rows of the run NaN: look at them all
+      bool odd = false;
+      for (int r = t; r < rows.y - rows.x; r += kSwWarps * 32) {
+        const unsigned d = slot_addr<NC>(win_a, sw_row_slot(r, n0));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) odd = odd || !isfinite(lds_f(d + 16 * c)) || !isfinite(lds_f(d + 16 * c + 8));
+      }
+      if (all_red_or(odd)) {
+        if (t == 0) *(volatile int*)&s_redo = 1;
+        redo_run<NC>(a.image, a.groups + g_first, aux, xb, a.R, n0, ncol, win_a, warp, lane);
+        if (t == 0) *(volatile int*)&s_redo = 0;
+      }
       if (!bad)
         for (int e = t; e < (rows.y - rows.x) * NC; e += kSwWarps * 32) {
           const int r = e / NC, c = e % NC;

@@ -483,7 +483,8 @@ struct Builder {
             const DenseOp& o = ops[B.rows[(size_t)ri].op];
             const int32_t r = B.rows[(size_t)ri].row, nin = o.nin();
             const int32_t lo = (l & (G - 1)) * E, hi = std::min<int32_t>(nin, lo + E);   // the lane's inputs
-            b = o.in0 + std::min(lo, even(nin));
+            // within the op's own slots; a lane longer than the op goes on within the region
+            b = o.in0 + std::max(0, std::min(lo, even(nin) - E));
             b = std::max(B.reg_lo, std::min(b, B.reg_hi - E));
             for (int32_t i = lo; i < hi; ++i) w[(size_t)(o.in0 + i - b)] = o.coef[(size_t)r * nin + i];
             if ((l & (G - 1)) == 0) {

@@ -8,10 +8,12 @@
 // executed with the kernel's input rule, is off the packed program's sweep by more than 1e-5.
 //
 // CHECK = nan, nan_small (the smallest resident window): a NaN in one row of the second of a CTA's two right-hand sides, the shared
-// memory of the kernel followed byte by byte (window, gather slices, entry pairs; triangles
-// masked at the diagonal).  Fails where the first right-hand side is not finite throughout, or
-// the second one in other rows than the packed program's sweep gives.  Rows: a few at the edges
-// of leaves and of the resident runs.
+// memory of the kernel followed byte by byte (window, gather slices, entry pairs; a run whose
+// rows come out non-finite once more with the zero coefficients masked).  Fails where the first
+// right-hand side changes, or the second one is finite in other rows than the packed program's
+// sweep.  Also with a value whose products overflow in place of the NaN: fails where the first
+// right-hand side changes, or rows of the second one that do not depend on the value.  Rows: a
+// few at the edges of leaves and of the resident runs.
 //
 //   sweepcheck triangle
 //
@@ -118,6 +120,7 @@ struct Cta {
     float v[NC][2];
   };
   std::vector<Out> outs;   // of the current phase, stored when it ends
+  int batch = 0;           // of the current global phase
 
   Cta(const PackedHost& p, const SwSched& s) : ph(p), S(s) {
     for (auto& v : st) v.assign((size_t)ph.state_len, 0.f);
@@ -126,7 +129,8 @@ struct Cta {
   std::complex<float>& global(int32_t s, int c) { return s < ph.n ? x[c][(size_t)s] : st[c][(size_t)(s - ph.n)]; }
 
   // sums of one row: its lanes' entries over pairs that start at float `base` of the window
-  void row(const SwDesc& D, const uint8_t* d, int t, int i, int64_t t0, int elen, bool res, size_t base, float (&v)[NC][2]) {
+  void row(const SwDesc& D, const uint8_t* d, int t, int i, int64_t t0, int elen, bool res, size_t base, bool mask,
+           float (&v)[NC][2]) {
     const float* cf = reinterpret_cast<const float*>(d + D.off_coef);
     const int16_t* in = reinterpret_cast<const int16_t*>(d + D.off_in);
     for (int c = 0; c < NC; ++c) {
@@ -137,6 +141,7 @@ struct Cta {
           const int e2 = res && e < 2 * kSwTilePairs ? 2 * sw_tile_pair(e / 2, elen / 2) : e;
           const float* w = win.data() + base + (size_t)(in[32 * t + l] + e2) / 2 * 4 * NC + 4 * c;
           for (int q = 0; q < 2; ++q) {
+            if (mask && m[q] == 0.f && m[2 + q] == 0.f) continue;
             re += m[q] * w[q] - m[2 + q] * w[2 + q];
             im += m[q] * w[2 + q] + m[2 + q] * w[q];
           }
@@ -145,8 +150,9 @@ struct Cta {
       v[c][1] = im;
     }
   }
-  void triangle(const SwDesc& D, const uint8_t* d, bool up) {
+  void triangle(const SwDesc& D, const uint8_t* d, bool up, bool mask) {
     const int s = D.nrows, n0 = (int)ph.n0;
+    mask = mask || (n0 & 1);
     std::vector<float> out((size_t)s * NC * 2, 0.f);
     for (int v = 0; v < sw_tri_warps(s); ++v) {
       const int32_t tw = reinterpret_cast<const int32_t*>(d)[v];
@@ -155,10 +161,11 @@ struct Cta {
         for (int q = 0; q < 16; ++q) {
           const int j = 4 * v + q / 4, r = i < n1 ? s - 1 - j : j, p = q % 4 + 4 * (i < n1 ? i : i - n1);
           if (!sw_tri_live(s, j, i < n1)) continue;
+          if (!mask && p / 4 >= sw_tri_take(s, p % 4, i < n1 ? n1 : nn0)) continue;
           const float* m = reinterpret_cast<const float*>(d + kSwTriTab) + ((int64_t)((tw >> 16) + i) * 32 + 2 * q) * 2;
           for (int u = 0; u < 2; ++u) {
             const int c0 = (up ? s - 2 - 2 * p : 2 * p) + u, row = up ? s - 1 - r : r;
-            if (c0 < 0 || c0 >= s || (up ? c0 < row : c0 > row)) continue;
+            if (mask && (c0 < 0 || c0 >= s || (up ? c0 < row : c0 > row))) continue;
             for (int c = 0; c < NC; ++c) {
               const float* w = slot(D.a0 + sw_row_slot(c0, n0), c);
               out[((size_t)row * NC + c) * 2] += m[u] * w[0] - m[2 + u] * w[2];
@@ -174,80 +181,95 @@ struct Cta {
         w[2] = out[((size_t)r * NC + c) * 2 + 1];
       }
   }
-  void sweep() {
+  void group(const SwGroup& G, bool mask) {
     const int n0 = (int)ph.n0;
-    int batch = 0;   // of the current global phase
-    for (const SwGroup& G : S.groups) {
-      const uint8_t* gb = S.image.data() + G.img;
-      SwGroupHdr H;
-      std::memcpy(&H, gb, sizeof(H));
-      const bool res = (H.flags & SWG_RES) != 0;
-      if (H.flags & SWG_BEGIN) {
-        std::fill(win.begin(), win.begin() + (H.flags >> kSwGroupSlots) * 2 * NC, 0.f);
-        for (int32_t r = 0; r < H.beg_hi - H.beg_lo; ++r)
-          for (int c = 0; c < NC; ++c) {
-            float* w = slot(sw_row_slot(r, n0), c);
-            w[0] = x[c][(size_t)(H.beg_lo + r)].real();
-            w[2] = x[c][(size_t)(H.beg_lo + r)].imag();
-          }
-      }
-      int64_t di = 0;
-      for (int k = 0; k < H.nph; ++k) {
-        SwPhase PH;
-        std::memcpy(&PH, gb + 32 + 8 * k, sizeof(PH));
-        for (int b = 0; b < PH.nb; ++b, ++di) {
-          SwDesc D;
-          std::memcpy(&D, gb + H.off_desc + 40 * di, sizeof(D));
-          const uint8_t* d = gb + D.off;
-          if (PH.flags & SWP_TRI) { triangle(D, d, (PH.flags & SWP_UPPER) != 0); continue; }
-          const int32_t* out = reinterpret_cast<const int32_t*>(d);
-          const int32_t* e0 = reinterpret_cast<const int32_t*>(d + D.off_e0);
-          const int32_t* gl = reinterpret_cast<const int32_t*>(d + D.off_gl);
-          const size_t raw = (size_t)(batch % kSwWarps) * (2 * kSwGather * NC * 2), pairs = raw + kSwGather * NC * 2;
-          if (!res) {
-            for (int q = 0; q < D.ngl; ++q)
-              for (int c = 0; c < NC; ++c) {
-                const std::complex<float> v = gl[q] < 0 ? 0.f : global(gl[q], c);
-                win[raw + (size_t)q * 2 * NC + 2 * c] = v.real();
-                win[raw + (size_t)q * 2 * NC + 2 * c + 1] = v.imag();
-              }
-            for (int q = 0; 2 * q < (D.a0 > 0 ? D.a0 : D.ngl); ++q) {
-              float e[2][NC][2];
-              std::memcpy(e, &win[raw + (size_t)q * 4 * NC], sizeof(e));
-              float* p = &win[pairs + (size_t)q * 4 * NC];
-              for (int c = 0; c < NC; ++c)
-                for (int u = 0; u < 2; ++u) { p[4 * c + u] = e[u][c][0]; p[4 * c + 2 + u] = e[u][c][1]; }
-            }
-            ++batch;
-          }
-          const int rpt = 32 >> D.glog;
-          for (int r = 0; r < D.nrows; ++r) {
-            const int t = r / rpt;
-            Out o{out[r], {}};
-            row(D, d, t, r % rpt, res ? 0 : 32 * (int64_t)e0[t], res ? D.elen : e0[t + 1] - e0[t], res, res ? 0 : pairs, o.v);
-            if (!res && D.a0)
-              for (int c = 0; c < NC; ++c)
-                for (int u = 0; u < 2; ++u) o.v[c][u] += win[raw + (size_t)(D.a0 + r) * 2 * NC + 2 * c + u];
-            outs.push_back(o);
-          }
+    const uint8_t* gb = S.image.data() + G.img;
+    SwGroupHdr H;
+    std::memcpy(&H, gb, sizeof(H));
+    const bool res = (H.flags & SWG_RES) != 0;
+    if (H.flags & SWG_BEGIN) {
+      std::fill(win.begin(), win.begin() + (H.flags >> kSwGroupSlots) * 2 * NC, 0.f);
+      for (int32_t r = 0; r < H.beg_hi - H.beg_lo; ++r)
+        for (int c = 0; c < NC; ++c) {
+          float* w = slot(sw_row_slot(r, n0), c);
+          w[0] = x[c][(size_t)(H.beg_lo + r)].real();
+          w[2] = x[c][(size_t)(H.beg_lo + r)].imag();
         }
-        if (!(PH.flags & SWP_END)) continue;
-        for (const Out& o : outs)
-          for (int c = 0; c < NC; ++c) {
-            if (!res) { global(o.o, c) = {o.v[c][0], o.v[c][1]}; continue; }
-            float* w = slot(o.o & ~kSwAcc, c);
-            w[0] = ((o.o & kSwAcc) ? w[0] : 0.f) + o.v[c][0];
-            w[2] = ((o.o & kSwAcc) ? w[2] : 0.f) + o.v[c][1];
+    }
+    int64_t di = 0;
+    for (int k = 0; k < H.nph; ++k) {
+      SwPhase PH;
+      std::memcpy(&PH, gb + 32 + 8 * k, sizeof(PH));
+      for (int b = 0; b < PH.nb; ++b, ++di) {
+        SwDesc D;
+        std::memcpy(&D, gb + H.off_desc + 40 * di, sizeof(D));
+        const uint8_t* d = gb + D.off;
+        if (PH.flags & SWP_TRI) { triangle(D, d, (PH.flags & SWP_UPPER) != 0, mask); continue; }
+        const int32_t* out = reinterpret_cast<const int32_t*>(d);
+        const int32_t* e0 = reinterpret_cast<const int32_t*>(d + D.off_e0);
+        const int32_t* gl = reinterpret_cast<const int32_t*>(d + D.off_gl);
+        const size_t raw = (size_t)(batch % kSwWarps) * (2 * kSwGather * NC * 2), pairs = raw + kSwGather * NC * 2;
+        if (!res) {
+          for (int q = 0; q < D.ngl; ++q)
+            for (int c = 0; c < NC; ++c) {
+              const std::complex<float> v = gl[q] < 0 ? 0.f : global(gl[q], c);
+              win[raw + (size_t)q * 2 * NC + 2 * c] = v.real();
+              win[raw + (size_t)q * 2 * NC + 2 * c + 1] = v.imag();
+            }
+          for (int q = 0; 2 * q < (D.a0 > 0 ? D.a0 : D.ngl); ++q) {
+            float e[2][NC][2];
+            std::memcpy(e, &win[raw + (size_t)q * 4 * NC], sizeof(e));
+            float* p = &win[pairs + (size_t)q * 4 * NC];
+            for (int c = 0; c < NC; ++c)
+              for (int u = 0; u < 2; ++u) { p[4 * c + u] = e[u][c][0]; p[4 * c + 2 + u] = e[u][c][1]; }
           }
-        outs.clear();
-        batch = 0;
+          ++batch;
+        }
+        const int rpt = 32 >> D.glog;
+        for (int r = 0; r < D.nrows; ++r) {
+          const int t = r / rpt;
+          Out o{out[r], {}};
+          row(D, d, t, r % rpt, res ? 0 : 32 * (int64_t)e0[t], res ? D.elen : e0[t + 1] - e0[t], res, res ? 0 : pairs, mask, o.v);
+          if (!res && D.a0)
+            for (int c = 0; c < NC; ++c)
+              for (int u = 0; u < 2; ++u) o.v[c][u] += win[raw + (size_t)(D.a0 + r) * 2 * NC + 2 * c + u];
+          outs.push_back(o);
+        }
       }
-      if (H.flags & SWG_ENDRUN)
-        for (int32_t r = 0; r < H.end_hi - H.end_lo; ++r)
-          for (int c = 0; c < NC; ++c) {
-            const float* w = slot(sw_row_slot(r, n0), c);
-            x[c][(size_t)(H.end_lo + r)] = {w[0], w[2]};
-          }
+      if (!(PH.flags & SWP_END)) continue;
+      for (const Out& o : outs)
+        for (int c = 0; c < NC; ++c) {
+          if (!res) { global(o.o, c) = {o.v[c][0], o.v[c][1]}; continue; }
+          float* w = slot(o.o & ~kSwAcc, c);
+          w[0] = ((o.o & kSwAcc) ? w[0] : 0.f) + o.v[c][0];
+          w[2] = ((o.o & kSwAcc) ? w[2] : 0.f) + o.v[c][1];
+        }
+      outs.clear();
+      batch = 0;
+    }
+  }
+  void sweep() {
+    size_t begin = 0;
+    for (size_t g = 0; g < S.groups.size(); ++g) {
+      SwGroupHdr H;
+      std::memcpy(&H, S.image.data() + S.groups[g].img, sizeof(H));
+      if (H.flags & SWG_BEGIN) begin = g;
+      group(S.groups[g], false);
+      if (!(H.flags & SWG_ENDRUN)) continue;
+      const int rows = H.end_hi - H.end_lo;
+      bool odd = false;
+      for (int r = 0; r < rows; ++r)
+        for (int c = 0; c < NC; ++c) {
+          const float* w = slot(sw_row_slot(r, (int)ph.n0), c);
+          odd = odd || !std::isfinite(w[0]) || !std::isfinite(w[2]);
+        }
+      if (odd)
+        for (size_t q = begin; q <= g; ++q) group(S.groups[q], true);
+      for (int r = 0; r < rows; ++r)
+        for (int c = 0; c < NC; ++c) {
+          const float* w = slot(sw_row_slot(r, (int)ph.n0), c);
+          x[c][(size_t)(H.end_lo + r)] = {w[0], w[2]};
+        }
     }
   }
 };
@@ -261,24 +283,33 @@ int nan(const PackedHost& ph, int win_slots) {
     SwSched S;
     build_sweep_sched(ph, which, 8, win_slots, S);
     if (!S.ok) { std::printf("FAIL: no schedule: %s\n", S.why); return 1; }
+    const auto run = [&](int64_t at, float value) {
+      Cta cta(ph, S);
+      for (auto& v : cta.x) v.assign(b.begin(), b.end());
+      if (at >= 0) cta.x[1][(size_t)at] = value;
+      cta.sweep();
+      return cta;
+    };
+    const Cta clean = run(-1, 0);
+    const bool up = which == 1 || which == 2;   // rows from the last one on
     for (int64_t at : {(int64_t)5, n0 - 1, n0, n0 + 3, 5 * n0 + n0 / 2, n / 2 - 1, n / 2, n / 2 + n0 + 1, n - n0, n - 2}) {
       std::vector<cplx> ref = b;
       ref[(size_t)at] = NAN;
-      Cta cta(ph, S);
-      for (auto& v : cta.x) v.assign(b.begin(), b.end());
-      cta.x[1][(size_t)at] = NAN;
-      cta.sweep();
       HostFactor none;
       host_sweep(ph, none, which, ref.data());
-      int64_t first = 0, second = 0;
-      for (int64_t r = 0; r < n; ++r) {
-        first += !finite(cta.x[0][(size_t)r]);
-        second += finite(cta.x[1][(size_t)r]) != finite(ref[(size_t)r]);
-      }
-      if (first || second) {
-        std::printf("FAIL: sweep %d, NaN at %lld: %lld rows of the other column, %lld rows of its own\n", which, (long long)at,
-                    (long long)first, (long long)second);
-        return 1;
+      for (float value : {NAN, 3e38f}) {
+        const Cta cta = run(at, value);
+        int64_t first = 0, free = 0, pattern = 0;
+        for (int64_t r = 0; r < n; ++r) {
+          first += cta.x[0][(size_t)r] != clean.x[0][(size_t)r];
+          if (up ? r > at : r < at) free += cta.x[1][(size_t)r] != clean.x[1][(size_t)r];
+          if (std::isnan(value)) pattern += finite(cta.x[1][(size_t)r]) != finite(ref[(size_t)r]);
+        }
+        if (first || free || pattern) {
+          std::printf("FAIL: sweep %d, %g at %lld: %lld rows of the other column, %lld independent rows, %lld rows\n", which,
+                      (double)value, (long long)at, (long long)first, (long long)free, (long long)pattern);
+          return 1;
+        }
       }
     }
   }

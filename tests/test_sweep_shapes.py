@@ -108,8 +108,9 @@ def test_sweep_leaves_off_a_multiple_of_eight_on_the_device(hb_gpu, n, leaf):
     _check_sweeps(hb_gpu, "arc", n, leaf, 1e-6)
 
 
-# (factors with global phases before resident runs)
-@pytest.mark.parametrize("check,n,leaf", [("nan", 16384, 64), ("nan_small", 1600, 25), ("nan_small", 1600, 50)])
+# (factors with global phases before resident runs; tiles whose lanes read past their op's inputs)
+@pytest.mark.parametrize("check,n,leaf", [("nan", 16384, 64), ("nan_small", 1600, 25), ("nan_small", 1600, 50),
+                                          ("nan", 1600, 50), ("nan", 2400, 75), ("nan_small", 2400, 75)])
 def test_nan_stays_in_its_column_by_the_kernels_rule(sweepcheck, check, n, leaf):
     sweepcheck(check, "arc", n, leaf, 1e-6)
 
@@ -131,3 +132,28 @@ def test_nan_stays_in_its_column_on_the_device(hb_gpu, n, leaf, row, small):
         clean, x = fn(f, b, op), fn(f, bad, op)
         assert torch.equal(x[others], clean[others])
         assert torch.isnan(torch.view_as_real(x[q, row])).any()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("small", [False, True])
+@pytest.mark.parametrize("n,leaf,row", [(1600, 25, 703), (1600, 50, 405), (2400, 75, 80), (1024, 64, 129), (4096, 64, 5)])
+def test_rows_that_do_not_depend_on_it_keep_their_values(hb_gpu, n, leaf, row, small):
+    # A NaN, and a value whose products overflow: rows before it (L~^{-1}, U~^{-H}) or after it
+    # (U~^{-1}, L~^{-H}) have the same sums in the same order: equal.
+    import torch
+    hb = hb_gpu
+    f = hb.hb_factor(_geom(hb, "arc", n), leaf, 1e-6, form=hb.HB_C64, options=hb.HB_OPT_SWEEP_WINDOW_MIN if small else 0)
+    hb.hb_set_sweep_kernel(f, 1)
+    for R in (3, 160):
+        b = torch.from_numpy(W.complex_gaussian(n, 90, R).T.copy()).cuda().to(torch.complex64)
+        for fn, op, before in [(hb.hb_lower_solve, 0, True), (hb.hb_upper_solve, 0, False), (hb.hb_lower_solve, 1, False),
+                               (hb.hb_upper_solve, 1, True)]:
+            clean = fn(f, b, op)
+            for value in (float("nan"), 3e38):
+                bad = b.clone()
+                bad[1, row] = complex(value, 0.0)
+                x = fn(f, bad, op)
+                free = slice(0, row) if before else slice(row + 1, n)
+                assert torch.equal(x[1, free], clean[1, free]), (R, op, before, value)
+                others = [r for r in range(R) if r != 1]
+                assert torch.equal(x[others], clean[others]), (R, op, before, value)
