@@ -484,32 +484,28 @@ __device__ __forceinline__ void run_batch(const SwArgs& a, unsigned desc, unsign
 // every lane has the same 17 steps at order 128, a step's coefficients are consecutive,
 // its inputs four neighbouring column pairs that all row pairs share, and a row's sum
 // needs two shuffle rounds and no other warp; one barrier separates the reads of the rows
-// from their replacement.  FAST: without masks; else inputs beyond a row's diagonal are masked
-// (0 times a foreign row's Inf would be NaN).  EVEN: the window's slots pair up like the columns
-// (even leaf size).
-template <int NC, bool EVEN>
+// from their replacement.  FAST, for an even leaf size (the window's slots pair up like the
+// columns): without masks; else, for any, inputs beyond a row's diagonal are masked (0 times a
+// foreign row's Inf would be NaN).
+template <int NC>
 __device__ __forceinline__ f2x2 tri_input(unsigned win, int a0, int s, bool up, int p, int c, int n0) {
-  if constexpr (EVEN) {
-    return lds_2(slot_addr<NC>(win, a0 + (up ? s - 2 - 2 * p : 2 * p)) + 16 * c);
-  } else {
-    // columns c0, c0 + 1 by themselves (a column outside the triangle is masked by the caller)
-    const int c0 = up ? s - 2 - 2 * p : 2 * p;
-    unsigned q[4] = {0, 0, 0, 0};
+  // columns c0, c0 + 1 by themselves (a column outside the triangle is masked by the caller)
+  const int c0 = up ? s - 2 - 2 * p : 2 * p;
+  unsigned q[4] = {0, 0, 0, 0};
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (c0 + u >= 0 && c0 + u < s) {
-        const unsigned d = slot_addr<NC>(win, a0 + sw_row_slot(c0 + u, n0)) + 16 * c;
-        q[u] = __float_as_uint(lds_f(d));
-        q[2 + u] = __float_as_uint(lds_f(d + 8));
-      }
-    f2x2 v;
-    v.a = q[0] | (f2x)q[1] << 32;
-    v.b = q[2] | (f2x)q[3] << 32;
-    return v;
-  }
+  for (int u = 0; u < 2; ++u)
+    if (c0 + u >= 0 && c0 + u < s) {
+      const unsigned d = slot_addr<NC>(win, a0 + sw_row_slot(c0 + u, n0)) + 16 * c;
+      q[u] = __float_as_uint(lds_f(d));
+      q[2 + u] = __float_as_uint(lds_f(d + 8));
+    }
+  f2x2 v;
+  v.a = q[0] | (f2x)q[1] << 32;
+  v.b = q[2] | (f2x)q[3] << 32;
+  return v;
 }
 // row r's sum over steps [0, n) (r < 0: no such row); coef: the lane's first coefficient
-template <int NC, bool EVEN, class P>
+template <int NC, class P>
 __device__ __forceinline__ float2 tri_row(int n, P coef, int r, unsigned win, int a0, int s, bool up, int n0, int lane) {
   const int g = (lane >> 1) & 3, c = NC == 2 ? lane & 1 : 0;
   // with one column the lane takes every second step
@@ -520,7 +516,7 @@ __device__ __forceinline__ float2 tri_row(int n, P coef, int r, unsigned win, in
     const int p = g + 4 * i;
     const bool in = 2 * p <= r, two = 2 * p < r;   // the pair's first / second stored column within the row
     f2x2 v{0, 0};
-    if (in) v = tri_input<NC, EVEN>(win, a0, s, up, p, c, n0);
+    if (in) v = tri_input<NC>(win, a0, s, up, p, c, n0);
     const f2x mask = two ? ~0ull : up ? 0xffffffffull << 32 : 0xffffffffull;
     v.a &= mask;
     v.b &= mask;
@@ -528,8 +524,8 @@ __device__ __forceinline__ float2 tri_row(int n, P coef, int r, unsigned win, in
   }
   return acc.sum();
 }
-// The same without masks, for an even leaf size (the coefficients beyond the diagonal are zero;
-// n: the steps within the triangle), two steps in flight.  vp: the lane's first input, dv: bytes
+// The same without masks (the coefficients beyond the diagonal are zero; n: the steps within
+// the triangle), two steps in flight.  vp: the lane's first input, dv: bytes
 // per step.
 template <int NC>
 __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, int dv, int lane) {
@@ -552,7 +548,7 @@ __device__ __forceinline__ float2 tri_row_fast(int n, unsigned cp, unsigned vp, 
   if (i < n) acc.add(lds_2(cp), lds_2(vp));
   return acc.sum();
 }
-template <int NC, bool EVEN, bool FAST, class P>
+template <int NC, bool FAST, class P>
 __device__ __forceinline__ void run_tri(int s, int a0, bool up, P T, unsigned win, int n0, int warp, int lane) {
   const int dv = (up ? -64 : 64) * NC, g = (lane >> 1) & 3;
   const unsigned vp = slot_addr<NC>(win, a0 + (up ? s - 2 : 0)) + (NC == 2 ? 16 * (lane & 1) : 0) + g * (dv / 4);
@@ -572,8 +568,8 @@ __device__ __forceinline__ void run_tri(int s, int a0, bool up, P T, unsigned wi
         s1 = tri_row_fast<NC>(sw_tri_take(s, g, n1), coef, vp, dv, lane);
         s0 = tri_row_fast<NC>(sw_tri_take(s, g, nn0), coef + n1 * 256, vp, dv, lane);
       } else {
-        s1 = tri_row<NC, EVEN>(n1, coef, r1, win, a0, s, up, n0, lane);
-        s0 = tri_row<NC, EVEN>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
+        s1 = tri_row<NC>(n1, coef, r1, win, a0, s, up, n0, lane);
+        s0 = tri_row<NC>(nn0, coef + n1 * 256, r0, win, a0, s, up, n0, lane);
       }
       // parting the sums over the lanes: a lane pair keeps one row, then one component
       constexpr int d1 = NC == 2 ? 2 : 1, d2 = 2 * d1;
@@ -589,7 +585,7 @@ __device__ __forceinline__ void run_tri(int s, int a0, bool up, P T, unsigned wi
       val[h] = w;
       if (r >= 0 && (NC == 2 || !(lane & 4))) {
         const int row = up ? s - 1 - r : r;
-        dst[h] = slot_addr<NC>(win, a0 + (EVEN ? row : sw_row_slot(row, n0))) + (NC == 2 ? 16 * (lane & 1) : 0) + (b2 ? 8 : 0);
+        dst[h] = slot_addr<NC>(win, a0 + (FAST ? row : sw_row_slot(row, n0))) + (NC == 2 ? 16 * (lane & 1) : 0) + (b2 ? 8 : 0);
       }
     }
   }
@@ -634,7 +630,7 @@ __device__ __forceinline__ void load_rows(const float2* xb, int64_t R, int lo, i
 // stand in global memory (the ring has moved on), the sums have the order of the run proper.
 template <int NC>
 __device__ __forceinline__ void redo_run(const uint8_t* image, const SwGroup* groups, int ngroup, const float2* xb, int64_t R,
-                                      int n0, int ncol, unsigned win, int warp, int lane) {
+                                         int n0, int ncol, unsigned win, int warp, int lane) {
   for (int g = 0; g < ngroup; ++g) {
     const uint8_t* img = image + groups[g].img;
     const SwGroupHdr H = *reinterpret_cast<const SwGroupHdr*>(img);
@@ -648,8 +644,7 @@ __device__ __forceinline__ void redo_run(const uint8_t* image, const SwGroup* gr
       if (PH.flags & SWP_TRI) {
         const uint8_t* T = img + desc->off;
         const bool up = (PH.flags & SWP_UPPER) != 0;
-        if (n0 & 1) run_tri<NC, false, false>(desc->nrows, desc->a0, up, T, win, n0, warp, lane);
-        else run_tri<NC, true, false>(desc->nrows, desc->a0, up, T, win, n0, warp, lane);
+        run_tri<NC, false>(desc->nrows, desc->a0, up, T, win, n0, warp, lane);   // (any leaf size)
       } else {
         for (int b = warp; b < PH.nb; b += kSwWarps) {
           const SwDesc& D = desc[b];
@@ -684,6 +679,13 @@ __device__ __forceinline__ void redo_run(const uint8_t* image, const SwGroup* gr
       if (PH.flags & SWP_END) all_sync();
     }
   }
+}
+
+// Out of line for one column (inlined, the spiral's solve takes 12.36 ms, not 12.07), inlined for
+// two (called, the spills around the call cost 1.1 ms of the 35.7 ms of 256 columns).
+__device__ __noinline__ void redo_run_1(const uint8_t* image, const SwGroup* groups, int ngroup, const float2* xb, int64_t R,
+                                        int n0, int ncol, unsigned win, int warp, int lane) {
+  redo_run<1>(image, groups, ngroup, xb, R, n0, ncol, win, warp, lane);
 }
 
 template <int NC>
@@ -898,8 +900,8 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
             if (!bad) {
               const int toff = lds_i(desc), s = lds_i(desc + 8), a0 = lds_i(desc + 20);
               const bool up = (PH.y & SWP_UPPER) != 0;
-              if (n0 & 1) run_tri<NC, false, false>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
-              else run_tri<NC, true, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+              if (n0 & 1) run_tri<NC, false>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
+              else run_tri<NC, true>(s, a0, up, gimg + toff, win_a, n0, warp, lane);
             } else {
               all_sync();   // the barrier inside the triangle product
             }
@@ -940,7 +942,8 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
       }
       if (all_red_or(odd)) {
         if (t == 0) *(volatile int*)&s_redo = 1;
-        redo_run<NC>(a.image, a.groups + g_first, aux, xb, a.R, n0, ncol, win_a, warp, lane);
+        if constexpr (NC == 1) redo_run_1(a.image, a.groups + g_first, aux, xb, a.R, n0, ncol, win_a, warp, lane);
+        else redo_run<NC>(a.image, a.groups + g_first, aux, xb, a.R, n0, ncol, win_a, warp, lane);
         if (t == 0) *(volatile int*)&s_redo = 0;
       }
       if (!bad)
