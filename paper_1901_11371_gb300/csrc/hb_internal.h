@@ -476,6 +476,10 @@ constexpr int kSwMaxCols = 2;                // right-hand sides per CTA
 constexpr int kSwWinSlots = kSwWinBytes / (kSwMaxCols * 8);   // window slots (complex-FP32 entries per column)
 constexpr int kSwGather = kSwWinSlots / (2 * kSwWarps);       // gathered inputs of a global batch (a warp's slice: as
                                                               // gathered, and regrouped in pairs)
+// In a phase with an op above kSwGather inputs (SWG_WIDE) a list may take the whole slice, up to
+// twice as many: it is regrouped where it stands, and the next batch's inputs are not gathered
+// meanwhile.
+constexpr int kSwGatherMax = 2 * kSwGather;
 constexpr int kSwGroupBytes = 40 * 1024;     // target bytes of a group
 constexpr int kSwMaxPhases = 64;             // phases of one group
 constexpr int kSwFlight = 64;                // slots of groups (arrival and release barriers)
@@ -488,6 +492,7 @@ enum SwGroupFlag : int32_t {
   SWG_RES = 4,      // group: batches on the window
   SWG_BEGIN = 8,    // group: load the window rows of vector rows [beg_lo, beg_hi) first
   SWG_ENDRUN = 16,  // group: write vector rows [end_lo, end_hi) back after its last phase
+  SWG_WIDE = 32,    // first group of a global phase: lists of up to kSwGatherMax entries
 };
 // SwGroupHdr::flags of a run's first group, upper bits: the window slots that the run uses (rows,
 // then state).  The run starts with all of them written, those without a row with zeros: tiles

@@ -765,8 +765,8 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
     __syncwarp();
   } else {
     const int t = threadIdx.x;
-    // gather area of global batches: entries as gathered, then the same in pairs
-    const unsigned raw = win_a + warp * (2 * kSwGather * NC * 8), pairs = raw + kSwGather * NC * 8;
+    // gather area of global batches: entries as gathered, then the same in pairs (a long list in place)
+    const unsigned raw = win_a + warp * (kSwGatherMax * NC * 8);
     const bool vec16 = NC == 2 && (a.R % 2) == 0 && (lb % 2) == 0;
     // bounded wait for group g; its image is then at group_at(g)
     auto wait_group = [&](int g) -> bool {
@@ -808,6 +808,8 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
         // current one is computed from its regrouped inputs, if that group has arrived -- but for
         // rows that add, whose old values are still read from the gathered entries.
         const int gend = g + aux;
+        const bool wide = (H.y & SWG_WIDE) != 0;   // lists regrouped in place, one at a time
+        const unsigned pairs = raw + (wide ? 0 : kSwGather * NC * 8);
         if (warp > 0) release(g, 1);   // (the first group: its owner, and every warp that read its header)
         auto gather = [&](unsigned img, unsigned cd) {
           const int ngl = lds_i(cd + 16);
@@ -839,7 +841,7 @@ __global__ void __launch_bounds__(640, 1) k_sweep_cols(SwArgs a) {
           const int old0 = lds_i(cd + 20);
           regroup(old0 > 0 ? old0 : lds_i(cd + 16));
           const int nq = q + kSwWarps;
-          ahead = old0 == 0 && nq < gend &&
+          ahead = old0 == 0 && !wide && nq < gend &&
                   __all_sync(0xffffffffu, mb_test_wait(&s_mbar[nq % kSwFlight], (unsigned)nq / kSwFlight & 1u));
           if (ahead) {
             const unsigned ni = group_at(nq);

@@ -576,6 +576,47 @@ struct Builder {
     return best;
   }
 
+  // Ops with more inputs than a slice holds, cut by rows into ops over the inputs that those
+  // rows use (an ID's row uses one of the k skeletons: the other k - 1 columns are zero).
+  void split_wide_ops() {
+    std::vector<DenseOp> out;
+    for (DenseOp& op : ops) {
+      if (even(op.nin()) + (op.add ? 2 : 0) <= kSwGatherMax) { out.push_back(std::move(op)); continue; }
+      const int32_t nin = op.nin();
+      std::vector<char> use((size_t)nin, 0);
+      int32_t r0 = 0, nuse = 0;
+      auto emit = [&](int32_t r1) {
+        DenseOp B;
+        B.add = op.add;
+        for (int32_t i = 0; i < nin; ++i)
+          if (use[(size_t)i]) B.in.push_back(op.in[(size_t)i]);
+        for (int32_t r = r0; r < r1; ++r) {
+          B.out.push_back(op.out[(size_t)r]);
+          for (int32_t i = 0; i < nin; ++i)
+            if (use[(size_t)i]) B.coef.push_back(op.coef[(size_t)r * nin + i]);
+        }
+        out.push_back(std::move(B));
+        std::fill(use.begin(), use.end(), 0);
+        nuse = 0;
+        r0 = r1;
+      };
+      for (int32_t r = 0; r < op.rows(); ++r) {
+        const cplx* w = op.coef.data() + (size_t)r * nin;
+        auto fresh = [&] {
+          int32_t n = 0;
+          for (int32_t i = 0; i < nin; ++i) n += !use[(size_t)i] && w[i] != cplx(0.0, 0.0);
+          return n;
+        };
+        if (r > r0 && even(nuse + fresh()) + (op.add ? 2 : 0) > kSwGatherMax) emit(r);
+        nuse += fresh();
+        for (int32_t i = 0; i < nin; ++i)
+          if (w[i] != cplx(0.0, 0.0)) use[(size_t)i] = 1;
+      }
+      emit(op.rows());
+    }
+    ops.swap(out);
+  }
+
   void batches_of_phase(bool res, int32_t reg_lo, int32_t reg_hi, std::vector<PBatch>& bs) {
     bs.clear();
     std::vector<RowRef> order;
@@ -598,7 +639,9 @@ struct Builder {
     }
     // wide phase: consecutive ops, batches of about a forty-eighth of the phase (three per
     // compute warp; 3 to 8 KB of coefficients, so that a dozen fit the staging ring) with at
-    // most kSwGather inputs; an op whose rows exceed that is split by rows
+    // most kSwGather inputs (an op with more: kSwGatherMax, by itself); an op whose rows exceed
+    // that is split by rows
+    split_wide_ops();
     int64_t tot = 0;
     for (const DenseOp& o : ops) tot += (int64_t)o.rows() * even(o.nin()) * cb;
     const int64_t target = std::max<int64_t>(3072, std::min<int64_t>(8192, tot / (3 * kSwWarps)));
@@ -623,7 +666,8 @@ struct Builder {
     for (size_t o = 0; o < ops.size(); ++o) {
       DenseOp& op = ops[o];
       const int32_t nin = op.nin(), ne = even(nin);
-      if (ne + (op.add ? 2 : 0) > kSwGather) { S.ok = false; S.why = "an op has too many inputs"; return; }
+      const int32_t cap = ne + (op.add ? 2 : 0) > kSwGather ? kSwGatherMax : kSwGather;
+      if (nin < 1 || ne + (op.add ? 2 : 0) > cap) { S.ok = false; S.why = "an op's inputs"; return; }
       const int64_t rb = (int64_t)ne * cb + 8;
       // an op opens a new batch when its rows would overfill the current one
       const int64_t slots = (int64_t)cur.gl.size() + ne + (op.add ? (int64_t)cur.rows.size() + op.rows() + 1 : 0);
@@ -631,8 +675,8 @@ struct Builder {
       // rows per batch of a large op (every batch gathers the op's inputs again; its
       // position in the slice is 0 there)
       int32_t per = (int32_t)std::max<int64_t>(8, target / rb);
-      if (op.add) per = std::min(per, (kSwGather - ne) & ~1);
-      const bool split = op.rows() > 2 * per || (op.add && ne + op.rows() + 1 > kSwGather);
+      if (op.add) per = std::min(per, (cap - ne) & ~1);
+      const bool split = op.rows() > 2 * per || (op.add && ne + op.rows() + 1 > cap);
       if (split) close();
       for (int32_t r = 0; r < op.rows(); ++r) {
         if (split && (int32_t)cur.rows.size() >= per) close();
@@ -780,11 +824,13 @@ void build_sweep_sched(const PackedHost& ph, int which, int coef_bytes, int win_
           S.res_phases++;
         } else {
           S.glob_phases++;
-          // the phase's first group tells how many it has
+          // the phase's first group tells how many it has, and whether a list exceeds half a slice
           uint8_t* hb = S.image.data() + S.groups[g0].img;
           SwGroupHdr H;
           std::memcpy(&H, hb, sizeof(H));
           H.aux = (int32_t)(S.groups.size() - g0);
+          for (const PBatch& B : bs)
+            if ((int64_t)B.gl.size() > kSwGather) H.flags |= SWG_WIDE;
           std::memcpy(hb, &H, sizeof(H));
         }
         if (more) bd.ops.swap(next);
@@ -961,6 +1007,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
   const int cb = S.coef_bytes;
   int64_t run_left = 0;   // groups of the current resident run still to come
   int64_t glob_left = 0;  // groups of the current global phase still to come
+  bool wide = false;      // its lists may take a whole slice
   int32_t win_rows = 0, run_slots = 0;   // window slots of the run's rows; all that it uses
   // per window slot: the last resident phase that wrote / read it (a resident
   // phase's batches run concurrently on the compute warps, so no slot may be
@@ -1007,6 +1054,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
       if (glob_left == 0) {
         if (H.aux < 1) return "global phase without its length";
         glob_left = H.aux;
+        wide = (H.flags & SWG_WIDE) != 0;
       }
       --glob_left;
       if ((glob_left == 0) != ((P0.flags & SWP_END) != 0)) return "end of a global phase";
@@ -1045,7 +1093,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
         const int64_t end = D.off + D.off_gl + (res ? 0 : al16(4 * (int64_t)D.ngl));
         if (end > G.bytes) return "batch outside the group";
         if (D.glog < 0 || D.glog > 5) return "lanes per row";
-        if (!res && (D.ngl < 0 || D.ngl > kSwGather || (D.ngl & 1))) return "gather list longer than a warp slice";
+        if (!res && (D.ngl < 0 || D.ngl > (wide ? kSwGatherMax : kSwGather) || (D.ngl & 1))) return "gather list longer than a warp slice";
         const uint8_t* bb = gb + D.off;
         const int32_t* out = (const int32_t*)bb;
         const int32_t* e0 = (const int32_t*)(bb + D.off_e0);

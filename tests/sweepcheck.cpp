@@ -1,7 +1,11 @@
 // Host checks of the column-partitioned sweep schedules over coarse and fine factors (test
 // helper; built by tests/test_sweep_shapes.py with g++ against the library's host code).
 //
-//   sweepcheck CHECK arc|strip n leaf eps
+//   sweepcheck CHECK arc|strip|strips8 n leaf eps     (strips8: eight parallel strips, 0.3 wavelengths apart)
+//
+// CHECK = wide: prints the longest gather list of a global batch with the smallest resident
+// window, the number of inputs of the longest op, and the number of sweeps with a schedule;
+// fails where a schedule is off the packed program's sweep by more than 1e-5.
 //
 // CHECK = tiles3: prints how many resident tiles have three entry pairs whose third pair is
 // not zero (all four sweeps), and fails where a schedule with complex-FP32 coefficients,
@@ -36,11 +40,11 @@ namespace {
 PackedHost pack(const char* curve, int64_t n, int64_t leaf, double eps) {
   Geometry g;
   const double len = n / 20.0;
-  const double arc[3] = {len / M_PI, 0.0, M_PI}, strip[4] = {0.0, 0.0, len, 0.0};
-  const bool a = !std::strcmp(curve, "arc");
+  const double arc[3] = {len / M_PI, 0.0, M_PI}, strip[4] = {0.0, 0.0, len, 0.0}, strips8[3] = {8.0, len / 8.0, 0.3};
+  const bool a = !std::strcmp(curve, "arc"), s8 = !std::strcmp(curve, "strips8");
   HostFactor hf;
   PackedHost ph;
-  if (build_geometry(a ? HB_ARC : HB_STRIP, a ? arc : strip, a ? 3 : 4, n, g) ||
+  if (build_geometry(a ? HB_ARC : s8 ? HB_PARALLEL_STRIPS : HB_STRIP, a ? arc : s8 ? strips8 : strip, a || s8 ? 3 : 4, n, g) ||
       build_factor(g, 1.0, 376.73, 1.781072, leaf, eps, 1, hf, 0)) {
     std::printf("FAIL: factor\n");
     std::exit(1);
@@ -80,6 +84,41 @@ void resident_tiles(const SwSched& S, Fn fn) {
   }
 }
 
+// relative distance of a schedule's sweep from the packed program's
+double distance(const PackedHost& ph, const SwSched& S, int which) {
+  std::vector<cplx> x = vec(ph.n), r = x;
+  host_sweep_sched(ph, S, x.data());
+  HostFactor none;
+  host_sweep(ph, none, which, r.data());
+  double e = 0, d = 0;
+  for (int64_t i = 0; i < ph.n; ++i) { e += std::norm(x[i] - r[i]); d += std::norm(r[i]); }
+  return std::sqrt(e / d);
+}
+
+int wide(const PackedHost& ph) {
+  int longest = 0, nin = 0, sweeps = 0;
+  for (const DItem& it : ph.items) nin = std::max(nin, (int)it.a_k[0] + it.a_k[1]);
+  for (int which = 0; which < 4; ++which) {
+    SwSched S;
+    build_sweep_sched(ph, which, 8, 512, S);
+    if (!S.ok) continue;
+    ++sweeps;
+    if (const char* bad = check_sweep_sched(ph, S); *bad) { std::printf("FAIL: %s\n", bad); return 1; }
+    for (const SwGroup& G : S.groups) {
+      const uint8_t* gb = S.image.data() + G.img;
+      SwGroupHdr H;
+      SwDesc D;
+      std::memcpy(&H, gb, sizeof(H));
+      std::memcpy(&D, gb + H.off_desc, sizeof(D));
+      if (!(H.flags & SWG_RES)) longest = std::max(longest, D.ngl);
+    }
+    const double e = distance(ph, S, which);
+    if (!(e <= 1e-5)) { std::printf("FAIL: sweep %d off by %.3g\n", which, e); return 1; }
+  }
+  std::printf("list %d inputs %d sweeps %d\n", longest, nin, sweeps);
+  return 0;
+}
+
 int tiles3(const PackedHost& ph) {
   int count = 0;
   for (int which = 0; which < 4; ++which) {
@@ -95,13 +134,8 @@ int tiles3(const PackedHost& ph) {
         for (int u = 0; u < 4; ++u) live = live || c[2 * sw_pos(4, l) + u] != 0.f;
       count += live;
     });
-    std::vector<cplx> x = vec(ph.n), r = x;
-    host_sweep_sched(ph, S, x.data());
-    HostFactor none;
-    host_sweep(ph, none, which, r.data());
-    double e = 0, d = 0;
-    for (int64_t i = 0; i < ph.n; ++i) { e += std::norm(x[i] - r[i]); d += std::norm(r[i]); }
-    if (!(std::sqrt(e / d) <= 1e-5)) { std::printf("FAIL: sweep %d off by %.3g\n", which, std::sqrt(e / d)); return 1; }
+    const double e = distance(ph, S, which);
+    if (!(e <= 1e-5)) { std::printf("FAIL: sweep %d off by %.3g\n", which, e); return 1; }
   }
   std::printf("tiles %d\n", count);
   return 0;
@@ -121,6 +155,7 @@ struct Cta {
   };
   std::vector<Out> outs;   // of the current phase, stored when it ends
   int batch = 0;           // of the current global phase
+  bool wide = false;       // its lists may take a whole slice
 
   Cta(const PackedHost& p, const SwSched& s) : ph(p), S(s) {
     for (auto& v : st) v.assign((size_t)ph.state_len, 0.f);
@@ -187,6 +222,7 @@ struct Cta {
     SwGroupHdr H;
     std::memcpy(&H, gb, sizeof(H));
     const bool res = (H.flags & SWG_RES) != 0;
+    if (!res && H.aux > 0) wide = (H.flags & SWG_WIDE) != 0;
     if (H.flags & SWG_BEGIN) {
       std::fill(win.begin(), win.begin() + (H.flags >> kSwGroupSlots) * 2 * NC, 0.f);
       for (int32_t r = 0; r < H.beg_hi - H.beg_lo; ++r)
@@ -208,7 +244,7 @@ struct Cta {
         const int32_t* out = reinterpret_cast<const int32_t*>(d);
         const int32_t* e0 = reinterpret_cast<const int32_t*>(d + D.off_e0);
         const int32_t* gl = reinterpret_cast<const int32_t*>(d + D.off_gl);
-        const size_t raw = (size_t)(batch % kSwWarps) * (2 * kSwGather * NC * 2), pairs = raw + kSwGather * NC * 2;
+        const size_t raw = (size_t)(batch % kSwWarps) * (kSwGatherMax * NC * 2), pairs = raw + (wide ? 0 : kSwGather * NC * 2);
         if (!res) {
           for (int q = 0; q < D.ngl; ++q)
             for (int c = 0; c < NC; ++c) {
@@ -347,6 +383,7 @@ int main(int argc, char** argv) {
   const std::string what = argv[1];
   const PackedHost ph = pack(argv[2], std::atoll(argv[3]), std::atoll(argv[4]), std::atof(argv[5]));
   if (what == "tiles3") return tiles3(ph);
+  if (what == "wide") return wide(ph);
   if (what == "nan") return nan(ph, kSwWinSlots);
   if (what == "nan_small") return nan(ph, 512);
   return 2;

@@ -1,6 +1,7 @@
 """Column-partitioned sweeps of factors whose phases or triangles take other shapes than the usual:
 coarse ones, whose phases are so small that tiles have fewer entries, and sweep leaves whose
-order is no multiple of eight; and what a NaN in one right-hand side reaches.
+order is no multiple of eight; ops with more inputs than half a gather slice holds; and what a
+NaN in one right-hand side reaches.
 
 Bounds: a schedule with complex-FP32 coefficients, executed by the kernel's input rule, and the
 device's sweeps reproduce the packed program's own sweep to 1e-5 relative (the storage rounding
@@ -59,6 +60,8 @@ def hb_gpu():
 
 
 def _geom(hb, curve, n):
+    if curve == "strips8":
+        return hb.hb_geometry(hb.HB_PARALLEL_STRIPS, (8.0, n / 20.0 / 8.0, 0.3), n)
     if curve == "strip":
         return hb.hb_geometry(hb.HB_STRIP, (0.0, 0.0, n / 20.0, 0.0), n)
     return hb.hb_geometry(hb.HB_ARC, (n / 20.0 / math.pi, 0.0, math.pi), n)
@@ -157,3 +160,20 @@ def test_rows_that_do_not_depend_on_it_keep_their_values(hb_gpu, n, leaf, row, s
                 assert torch.equal(x[1, free], clean[1, free]), (R, op, before, value)
                 others = [r for r in range(R) if r != 1]
                 assert torch.equal(x[others], clean[others]), (R, op, before, value)
+
+
+# eight close strips, with global phases whose ops have 206 to 256 inputs; 400 (cut by rows; the
+# scatter ops of the other two sweeps have rows of more than 384)
+@pytest.mark.parametrize("n,leaf,eps,least,sweeps", [(2048, 32, 1e-6, 193, 4), (2048, 64, 1e-6, 193, 4),
+                                                     (4096, 32, 1e-9, 193, 4), (4096, 64, 1e-6, 385, 2)])
+def test_ops_with_many_inputs_have_a_schedule(sweepcheck, n, leaf, eps, least, sweeps):
+    _, longest, _, inputs, _, built = sweepcheck("wide", "strips8", n, leaf, eps)
+    assert int(longest) > 192 and int(inputs) >= least and int(built) == sweeps
+    if sweeps == 4:
+        sweepcheck("nan_small", "strips8", n, leaf, eps)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,leaf,eps", [(2048, 32, 1e-6), (2048, 64, 1e-6), (4096, 32, 1e-9)])
+def test_ops_with_many_inputs_on_the_device(hb_gpu, n, leaf, eps):
+    _check_sweeps(hb_gpu, "strips8", n, leaf, eps, options=hb_gpu.HB_OPT_SWEEP_WINDOW_MIN)
