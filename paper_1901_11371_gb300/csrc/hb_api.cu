@@ -164,7 +164,12 @@ int upload_factor(const PackedHost& ph, const HostFactor& hf, const Geometry& g,
     // they need the factor pool and the sweep-leaf triangles, released after upload)
     SwSched S[4];
     std::thread th[4];
-    for (int w = 0; w < 4; ++w) th[w] = std::thread([&, w] { build_sweep_sched(ph, w, 8, df.sw_win, S[w]); });
+    for (int w = 0; w < 4; ++w)
+      th[w] = std::thread([&, w] {
+        build_sweep_sched(ph, w, 8, df.sw_win, S[w]);
+        // (0.03 s of 4 s at N = 262,144)
+        if (S[w].ok && *check_sweep_sched(ph, S[w])) S[w].ok = false;
+      });
     for (auto& t : th) t.join();
     for (int w = 0; w < 4; ++w) {
       if (!S[w].ok) continue;   // the cooperative kernel serves this sweep

@@ -1079,7 +1079,7 @@ const char* check_sweep_sched(const PackedHost& ph, const SwSched& S) {
           const int64_t s = D.nrows;
           if (s < 1 || s % n0) return "triangle order";
           if (D.off + kSwTriTab + (int64_t)sw_tri_steps((int)s) * 32 * cb > G.bytes) return "triangle outside the group";
-          if (sw_tri_warps((int)s) * 4 > kSwTriTab) return "triangle order";
+          if (sw_tri_warps((int)s) > 2 * kSwWarps) return "triangle order";   // (a warp takes two parts at most)
           int step = 0;
           for (int v = 0; v < sw_tri_warps((int)s); ++v) {
             const SwTriWarp tw = sw_tri_warp((int)s, v);

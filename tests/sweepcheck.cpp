@@ -3,6 +3,9 @@
 //
 //   sweepcheck CHECK arc|strip|strips8 n leaf eps     (strips8: eight parallel strips, 0.3 wavelengths apart)
 //
+// CHECK = region: fails unless the structural check refuses a schedule of which one tile reads past
+// the slots of its run, inside the window.
+//
 // CHECK = wide: prints the longest gather list of a global batch with the smallest resident
 // window, the number of inputs of the longest op, and the number of sweeps with a schedule;
 // fails where a schedule is off the packed program's sweep by more than 1e-5.
@@ -82,6 +85,22 @@ void resident_tiles(const SwSched& S, Fn fn) {
       }
     }
   }
+}
+
+int region(const PackedHost& ph) {
+  SwSched S;
+  build_sweep_sched(ph, 0, 8, kSwWinSlots, S);
+  SwGroupHdr H;
+  std::memcpy(&H, S.image.data() + S.groups[0].img, sizeof(H));
+  const int slots = H.flags >> kSwGroupSlots;
+  bool done = false;
+  resident_tiles(S, [&](const SwDesc& D, const uint8_t* data) {
+    if (!done) reinterpret_cast<int16_t*>(const_cast<uint8_t*>(data) + D.off_in)[0] = (int16_t)slots;
+    done = true;
+  });
+  const std::string got = check_sweep_sched(ph, S);
+  std::printf("%s\n", got.c_str());
+  return slots + 64 <= kSwWinSlots && got == "input slot" ? 0 : 1;
 }
 
 // relative distance of a schedule's sweep from the packed program's
@@ -383,6 +402,7 @@ int main(int argc, char** argv) {
   const std::string what = argv[1];
   const PackedHost ph = pack(argv[2], std::atoll(argv[3]), std::atoll(argv[4]), std::atof(argv[5]));
   if (what == "tiles3") return tiles3(ph);
+  if (what == "region") return region(ph);
   if (what == "wide") return wide(ph);
   if (what == "nan") return nan(ph, kSwWinSlots);
   if (what == "nan_small") return nan(ph, 512);

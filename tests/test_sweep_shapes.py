@@ -177,3 +177,7 @@ def test_ops_with_many_inputs_have_a_schedule(sweepcheck, n, leaf, eps, least, s
 @pytest.mark.parametrize("n,leaf,eps", [(2048, 32, 1e-6), (2048, 64, 1e-6), (4096, 32, 1e-9)])
 def test_ops_with_many_inputs_on_the_device(hb_gpu, n, leaf, eps):
     _check_sweeps(hb_gpu, "strips8", n, leaf, eps, options=hb_gpu.HB_OPT_SWEEP_WINDOW_MIN)
+
+
+def test_inputs_beyond_a_runs_slots_are_refused(sweepcheck):
+    sweepcheck("region", "strip", 1024, 64, 1e-6)
