@@ -383,10 +383,11 @@ __device__ void do_op(const SweepArgs& a, const FlatOp& f, char* buf, int64_t bu
   if (pl.once) g.sync();
 }
 
+__device__ __forceinline__ int tri_pairs(int s) { return (s + 1) / 2; }
 // Sweep-leaf product x = T b, T the packed triangle of order s of the op
 // (lower, or upper with FF_UPPER), column-packed.  Thread (pair j, group g)
 // owns rows j and s-1-j (together s+1 triangle entries, so every thread has
-// the same share) and sums the columns c = g, g + ngrp, ... of each row inside
+// the same share; the last pair of an odd order is its middle row) and sums the columns c = g, g + ngrp, ... of each row inside
 // the triangle; for a fixed column consecutive threads read consecutive
 // entries.  part: ngrp * s * RC partial sums; b: the s input rows (stride W,
 // columns of this pass); results replace the rows of out (stride Wo) after a
@@ -396,14 +397,14 @@ __device__ __forceinline__ void tri_pass(const F* Tm, int s, bool upper, const t
                                          typename CT<T>::t* out, int64_t Wo, int rc, typename CT<T>::t* part,
                                          const Grp& gt) {
   using C = typename CT<T>::t;
-  const int npair = s > 1 ? s / 2 : 1;
+  const int npair = tri_pairs(s);
   const int ngrp = gt.nt / npair > 0 ? gt.nt / npair : 1;
   for (int e = gt.t; e < ngrp * npair; e += gt.nt) {
     const int j = e % npair, g = e / npair;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = h == 0 ? j : s - 1 - j;
-      if (h == 1 && r == j) break;   // s == 1
+      if (h == 1 && r == j) break;   // the middle row of an odd order
       C acc[RC];
 #pragma unroll
       for (int rr = 0; rr < RC; ++rr) acc[rr] = z2<T>();
@@ -449,7 +450,7 @@ __device__ void do_leaf(const SweepArgs& a, const FlatOp& f, char* buf, int64_t 
   const F* Tg = (const F*)a.tinv + f.moff;
   C* v = (C*)a.vec + (int64_t)f.src0 * R;
   const bool upper = (f.flags & FF_UPPER) != 0;
-  const int npair = s > 1 ? s / 2 : 1;
+  const int npair = tri_pairs(s);
   const int ngrp = g.nt / npair > 0 ? g.nt / npair : 1;
   const int64_t mb = align16((int64_t)f.melems * (int64_t)sizeof(F));
   const int64_t partb = align16((int64_t)ngrp * s * RC * (int64_t)sizeof(C));
