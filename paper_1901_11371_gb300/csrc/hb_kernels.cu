@@ -824,9 +824,9 @@ __global__ void __launch_bounds__(kWThreads) k_wapply_exit(const DOuter* __restr
 // ---------------------------------------------------------------------------
 // Layout conversion kernels: column-major [R][ld] <-> [row][R] through a tile of
 // kTileRows rows x up to kTileCols columns in shared memory, so that both sides are
-// read and written along their contiguous index.  HBM-bound: 256 complex64 columns of
-// 262,144 rows take 0.17 ms (1.07 GB: 6.2 TB/s); element by element, with one side in
-// steps of ld, they took 1.1 ms.
+// read and written along their contiguous index; few columns go element by element
+// (below).  HBM-bound: 256 complex64 columns of 262,144 rows take 0.17 ms (1.07 GB:
+// 6.2 TB/s); element by element, with one side in steps of ld, they took 1.1 ms.
 // ---------------------------------------------------------------------------
 constexpr int kTileRows = 64, kTileCols = 32;
 // The tile of one CTA.  Column-major side: thread -> one row, every 4th column; row-major
@@ -910,25 +910,71 @@ __global__ void __launch_bounds__(256) k_residual_cols(const double2* b, int64_t
   }
 }
 
+// Few columns: element by element in the order of the row-major side, every thread busy (a tile
+// of few columns leaves most threads of its row-major side idle).  262,144 rows, us, element by
+// element against tiles: gather of complex128 3.8 / 19.8 (1 column), 15.0 / 22.1 (8), 18.5 / 23.5
+// (10), 22.1 / 24.6 (12), 28.8 / 27.1 (16); of complex64 4.9 / 13.9 (2), 13.9 / 15.1 (10),
+// 15.7 / 15.4 (12); the scatters meet at 16; residual 3.8 / 52.0 (1), 18.3 / 74.8 (8),
+// 45.4 / 94.9 (20), 115 / 100 (24).
+constexpr int kFewCols = 10, kFewResidual = 20;
+template <class T>
+__global__ void __launch_bounds__(256) k_gather_few(const T* __restrict__ src, int64_t ld, int64_t n, int64_t R,
+                                                    T* __restrict__ dst, double scale) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * R; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / R, c = e - row * R;
+    T v = src[c * ld + row];
+    if (scale != 1.0) v = T{(decltype(T::x))(scale * (double)v.x), (decltype(T::y))(scale * (double)v.y)};
+    dst[e] = v;
+  }
+}
+template <class T>
+__global__ void __launch_bounds__(256) k_scatter_few(const T* __restrict__ src, int64_t n, int64_t R, T* __restrict__ dst,
+                                                     int64_t ld) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * R; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / R, c = e - row * R;
+    dst[c * ld + row] = src[e];
+  }
+}
+__global__ void __launch_bounds__(256) k_residual_few(const double2* b, int64_t ld, const double2* __restrict__ y, int64_t n,
+                                                      int64_t R, double2* r) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * R; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / R, c = e - row * R;
+    const double2 u = b[c * ld + row], w = y[e];
+    r[c * ld + row] = {u.x - w.x, u.y - w.y};
+  }
+}
+static inline unsigned few_grid(int64_t total) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 32)); }
+
 static inline dim3 tile_grid(int64_t n, int64_t R) {
   const int64_t cb = (R + kTileCols - 1) / kTileCols;
   return dim3((unsigned)((n + kTileRows - 1) / kTileRows), (unsigned)(cb < 65535 ? cb : 65535));
 }
 
 int launch_gather_cols(const void* src, int t, int64_t ld, int64_t n, int64_t R, void* dst, double scale, cudaStream_t st) {
+  if (R <= kFewCols) {
+    if (t == 0) k_gather_few<<<few_grid(n * R), 256, 0, st>>>((const double2*)src, ld, n, R, (double2*)dst, scale);
+    else k_gather_few<<<few_grid(n * R), 256, 0, st>>>((const float2*)src, ld, n, R, (float2*)dst, scale);
+    return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
+  }
   const dim3 g = tile_grid(n, R);
   if (t == 0) k_gather_cols<<<g, 256, 0, st>>>((const double2*)src, ld, n, R, (double2*)dst, scale);
   else k_gather_cols<<<g, 256, 0, st>>>((const float2*)src, ld, n, R, (float2*)dst, scale);
   return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
 }
 int launch_scatter_cols(const void* src, int t, int64_t n, int64_t R, void* dst, int64_t ld, cudaStream_t st) {
+  if (R <= kFewCols) {
+    if (t == 0) k_scatter_few<<<few_grid(n * R), 256, 0, st>>>((const double2*)src, n, R, (double2*)dst, ld);
+    else k_scatter_few<<<few_grid(n * R), 256, 0, st>>>((const float2*)src, n, R, (float2*)dst, ld);
+    return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
+  }
   const dim3 g = tile_grid(n, R);
   if (t == 0) k_scatter_cols<<<g, 256, 0, st>>>((const double2*)src, n, R, (double2*)dst, ld);
   else k_scatter_cols<<<g, 256, 0, st>>>((const float2*)src, n, R, (float2*)dst, ld);
   return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
 }
 int launch_residual_cols(const void* b, int64_t ld, const void* y, int64_t n, int64_t R, void* r, cudaStream_t st) {
-  k_residual_cols<<<tile_grid(n, R), 256, 0, st>>>((const double2*)b, ld, (const double2*)y, n, R, (double2*)r);
+  if (R <= kFewResidual) k_residual_few<<<few_grid(n * R), 256, 0, st>>>((const double2*)b, ld, (const double2*)y, n, R, (double2*)r);
+  else k_residual_cols<<<tile_grid(n, R), 256, 0, st>>>((const double2*)b, ld, (const double2*)y, n, R, (double2*)r);
   return cudaGetLastError() == cudaSuccess ? HB_OK : HB_ECUDA;
 }
 
