@@ -30,7 +30,12 @@
 //     N = 65,536: 3,058 without, 1,699 with);
 //   * the resident phases alternate between two sets of eight warps: while one set
 //     computes, the other has its next coefficients in registers and waits only for
-//     the inputs; large phases and the sweep leaves are taken by all sixteen.
+//     the inputs; large phases and the sweep leaves are taken by all sixteen;
+//   * tiles and triangles also multiply zeros with slots that are not theirs, so that no
+//     lane needs a mask.  A run whose rows come out non-finite is repeated with every zero
+//     coefficient masked: an Inf or NaN reaches only the rows that depend on it.  (In a
+//     global phase it reaches what its butterfly writes, which is the same rows; a value that
+//     first overflows there may reach more of them.)
 // What bounds it is the dependent chain of one CTA: a phase costs 1,000 to 2,000
 // cycles (descriptor and coefficient fetch, the inputs' round trip, shuffles, a
 // barrier), far above its share of the 9 B/clk of staged data.

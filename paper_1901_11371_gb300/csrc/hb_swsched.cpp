@@ -213,7 +213,6 @@ struct Fuser {
     ops.resize((size_t)nc);
     // row of coefficients (over the component's inputs) of every state entry written so far
     std::vector<std::pair<int32_t, std::vector<cplx>>> val;   // (entry, row), found through at[]
-    std::vector<int32_t> touched;
     if (at.size() != (size_t)ph.state_len) at.assign((size_t)ph.state_len, -1);
     for (int32_t o = fp.base[p0]; o < fp.base[p0 + 1]; ++o) {
       const FlatOp& f = fp.ops[o];
